@@ -41,6 +41,8 @@ void set_error(const char* fmt, ...);
 // ahead on several streams.  Thread-safe.
 int ensure_smem(const void* fn, size_t bytes);
 
+constexpr int kSMs = 152;   // streaming multiprocessors of a GB300 (launch shaping only)
+
 // ----------------------------------------------------------------- index helpers
 
 __host__ __device__ inline int parity_p(int l) { return (l & 1) ? 0 : 1; }   // p_l

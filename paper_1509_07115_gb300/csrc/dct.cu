@@ -39,13 +39,13 @@ static InvKernel<R> inv_kernel(int N) {
 int dct_forward_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in,
                     double* out, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
-    unsigned th; size_t sm;
+    unsigned nb, th; size_t sm;
     FwdKernel<double> k = fwd_kernel<double, kPlain>(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);
-    int rc = launch_cfg(k, p->N, sizeof(double2), th, sm);
+    int rc = launch_cfg(k, p->N, nchannels(g), sizeof(double2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctFwd, st);
-    k<<<nblocks(g, p->N), th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, nullptr, nullptr, p->tw64, p->post64);
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, nullptr, nullptr, p->tw64, p->post64, fwd_scale<double>(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -53,13 +53,13 @@ int dct_forward_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const do
 int dct_forward_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const float* in,
                     float* out_hi, float* out_lo, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
-    unsigned th; size_t sm;
+    unsigned nb, th; size_t sm;
     FwdKernel<float> k = fwd_kernel<float, kSplitTF32>(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);
-    int rc = launch_cfg(k, p->N, sizeof(float2), th, sm);
+    int rc = launch_cfg(k, p->N, nchannels(g), sizeof(float2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctFwd, st);
-    k<<<nblocks(g, p->N), th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, nullptr, p->tw32, p->post32);
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, nullptr, p->tw32, p->post32, fwd_scale<float>(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -67,13 +67,13 @@ int dct_forward_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
 int dct_inverse_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in,
                     double* out, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
-    unsigned th; size_t sm;
+    unsigned nb, th; size_t sm;
     InvKernel<double> k = inv_kernel<double>(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);
-    int rc = launch_cfg(k, p->N, sizeof(double2), th, sm);
+    int rc = launch_cfg(k, p->N, nchannels(g), sizeof(double2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctInv, st);
-    k<<<nblocks(g, p->N), th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw64, p->post64);
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw64, p->post64, inv_scale<double>(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }

@@ -42,13 +42,13 @@ InvKernel<float> inv_kernel_f32(int N) {
 int dct_forward_f16(const dsbt_plan* p, const GroupTable& g, bool cplx, const float* in, __half* out_hi,
                     __half* out_lo, float* scale, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
-    unsigned th; size_t sm;
+    unsigned nb, th; size_t sm;
     FwdKernel<float> k = fwd_kernel_f16(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);
-    int rc = launch_cfg(k, p->N, sizeof(float2), th, sm);
+    int rc = launch_cfg(k, p->N, nchannels(g), sizeof(float2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctFwd, st);
-    k<<<nblocks(g, p->N), th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, scale, p->tw32, p->post32);
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, scale, p->tw32, p->post32, fwd_scale<float>(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -56,13 +56,13 @@ int dct_forward_f16(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
 int dct_inverse_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const float* in,
                     float* out, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
-    unsigned th; size_t sm;
+    unsigned nb, th; size_t sm;
     InvKernel<float> k = inv_kernel_f32(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);
-    int rc = launch_cfg(k, p->N, sizeof(float2), th, sm);
+    int rc = launch_cfg(k, p->N, nchannels(g), sizeof(float2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctInv, st);
-    k<<<nblocks(g, p->N), th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw32, p->post32);
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw32, p->post32, inv_scale<float>(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }

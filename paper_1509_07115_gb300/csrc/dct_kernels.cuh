@@ -36,6 +36,8 @@
 // TF32-split kernels for N = 2048, 4096, 8192 and per Q otherwise.
 #pragma once
 
+#include <math.h>
+
 #include <cuda_fp16.h>
 
 #include "plan.cuh"
@@ -144,7 +146,12 @@ __device__ __forceinline__ void stockham_stage(C* s, const C* __restrict__ tw, i
             for (int r = 0; r < RX; ++r) x[u][r] = s[padi(j + r * nb)];
         }
         if (k > 0) {
-            if (RX == 16) {
+            if (RX == 16 && sizeof(C) == 16) {
+                // FP64: a product of two table entries costs four instructions
+                // of the FP64 pipe (under two lanes per clock and SM), a load none
+#pragma unroll
+                for (int r = 1; r < 16; ++r) x[u][r] = cmul(x[u][r], tw[r * b]);
+            } else if (RX == 16) {
                 const C w1 = tw[b], w4 = tw[4 * b];
                 const C w2 = cmul(w1, w1), w3 = cmul(w2, w1), w8 = cmul(w4, w4), w12 = cmul(w8, w4);
                 const C lo[4] = {w1, w1, w2, w3};
@@ -336,8 +343,18 @@ template <> __device__ __forceinline__ void st_pair<double2>(double2* p, double2
 }
 
 // Lines per CTA: as many lines of N/16 threads as fit in 256 threads (one
-// line of up to 512 threads when N/16 > 256).
-__host__ __device__ inline int lines_per_cta(int N) { return (N / 16 >= 256) ? 1 : 256 / (N / 16); }
+// line of up to 512 threads when N/16 > 256), but no more than leave every SM
+// a CTA.  The FP64 transform is bound by the FP64 pipe (1.7 lanes per clock
+// and SM measured: about 48 operations per point, 30 us for a line of 2048
+// points on one SM), so a call of few channels is as slow as its fullest CTA:
+// 64 channels of 2048 points took 67 us with two lines per CTA and 33 us with
+// one, 32 channels of 1024 points 66 us (four per CTA) and 30 us.  Calls with
+// more channels than SMs keep the fuller CTAs.
+inline int lines_per_cta(int N, int nchan) {
+    const int most = (N / 16 >= 256) ? 1 : 256 / (N / 16);
+    const int even = (nchan + kSMs - 1) / kSMs;
+    return even < most ? even : most;
+}
 
 // Output modes of the forward transform (planar lines, storage index n - p_l):
 // kPlain: R values; kSplitTF32: the TF32 pair hi + lo as two FP32 lines;
@@ -348,6 +365,13 @@ __host__ __device__ inline int lines_per_cta(int N) { return (N / 16 >= 256) ? 1
 // follow far below the FP16 range (|v| <= ||v|| < 2^13.5) and puts the FP16
 // subnormal step (2^-24) 2^-36 below the channel norm.
 enum : int { kPlain = 0, kSplitTF32 = 1, kSplitF16 = 2 };
+
+// Scale factors of a transform, computed on the host: as per-thread square
+// roots and divisions in FP64 they cost as much as a radix-4 stage.
+template <typename R>
+struct DctScale {
+    R c0, c1;   // forward: sqrt(1/N), sqrt(2/N); inverse: 1/sqrt(N), 1/sqrt(2N), the unscaled FFT's 1/N in them
+};
 
 // Power-of-two exponent e with x 2^e in [2^12, 2^13) (0 for 0, inf, nan).
 __device__ __forceinline__ int scale_exp(float nrm) {
@@ -363,13 +387,13 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
                                                  void* __restrict__ out0, void* __restrict__ out1,
                                                  float* __restrict__ scale,
                                                  const typename Cx<R>::T* __restrict__ tw,
-                                                 const typename Cx<R>::T* __restrict__ post) {
+                                                 const typename Cx<R>::T* __restrict__ post, DctScale<R> dsc) {
     typedef typename Cx<R>::T C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float spart[32];   // per 16 threads (<= 512 threads): partial sums of |psi_i|^2
     const int N = NS ? NS : Nrt;
     const int T = N >> 4;
-    const int G = lines_per_cta(N);
+    const int G = blockDim.x / T;
     const int grp = threadIdx.x / T, lt = threadIdx.x % T;
     C* s = reinterpret_cast<C*>(smem_raw) + (size_t)grp * (N + (N >> 4));
     const int chan = blockIdx.x * G + grp;
@@ -436,7 +460,7 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
     __shared__ C sroot[32];
     fft_stages<Q, NS>(s, tw, sroot, N, lt, T, 1, N);
     if (!live) return;
-    const R sc1 = (R)sqrt(2.0 / (double)N), sc0 = (R)sqrt(1.0 / (double)N);
+    const R sc1 = dsc.c1, sc0 = dsc.c0;
     const int line = g.line0[gi] + (cplx ? 2 * local : local);
     float fs = 1.f;
     if (MODE == kSplitF16) {
@@ -448,6 +472,44 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
             scale[line] = ldexpf(1.f, -e);
             if (cplx) scale[line + 1] = ldexpf(1.f, -e);
         }
+    }
+    if (MODE == kPlain) {
+        // k and N - k together: with A = w V_k and B = conj(w) V_{N-k} (w_{N-k} =
+        // -i conj(w)), X_k = (A + B) / 2 and X_{N-k} = i (A - B) / 2: two
+        // products for two outputs, and half the shared-memory reads.
+        R* o0 = reinterpret_cast<R*>(out0) + (size_t)line * N;
+        const int stT = pstride(T);
+        const R half = (R)0.5 * sc1;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {   // k = lt + i T < N / 2 = 8 T
+            const int k = lt + i * T;
+            C X0, X1;
+            int k1 = N - k;
+            if (k == 0) {   // its own partner; this thread also takes k = N / 2
+                const C v0 = s[0], vh = s[padi(N / 2)];
+                const R h = (R)0.70710678118654752440 * sc1;
+                X0.x = v0.x * sc0; X0.y = v0.y * sc0;
+                X1.x = vh.x * h;   X1.y = vh.y * h;
+                k1 = N / 2;
+            } else {
+                const C a = NS > 0 ? s[padi(lt) + i * stT] : s[padi(k)];
+                const C b = NS > 0 ? s[padi(N - lt) - i * stT] : s[padi(N - k)];
+                C w = post[k];
+                w.x *= half; w.y *= half;
+                const C A = cmul(a, w), B = cmulc(b, w);
+                X0 = cadd(A, B);
+                const C D = csub(A, B);
+                X1.x = -D.y; X1.y = D.x;
+            }
+            const int i0 = even ? N - 1 - k : k, i1 = even ? N - 1 - k1 : k1;
+            o0[i0] = X0.x;
+            o0[i1] = X1.x;
+            if (cplx) {
+                o0[N + i0] = X0.y;
+                o0[N + i1] = X1.y;
+            }
+        }
+        return;
     }
     const int st2 = pstride(2 * T);
 #pragma unroll
@@ -500,14 +562,6 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
                 *reinterpret_cast<__half2*>(o1 + N + idx) = __float22half2_rn(
                     make_float2(vi.x - __low2float(hi2), vi.y - __high2float(hi2)));
             }
-        } else {
-            R* o0 = reinterpret_cast<R*>(out0) + (size_t)line * N;
-            o0[idx] = lo_e.x;
-            o0[idx + 1] = hi_e.x;
-            if (cplx) {
-                o0[N + idx] = lo_e.y;
-                o0[N + idx + 1] = hi_e.y;
-            }
         }
     }
 }
@@ -516,12 +570,12 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
 template <typename R, int Q, int NS>
 __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTable g, int Nrt, int cplx, const R* __restrict__ in,
                                                  R* __restrict__ out, const typename Cx<R>::T* __restrict__ tw,
-                                                 const typename Cx<R>::T* __restrict__ post) {
+                                                 const typename Cx<R>::T* __restrict__ post, DctScale<R> dsc) {
     typedef typename Cx<R>::T C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = NS ? NS : Nrt;
     const int T = N >> 4;
-    const int G = lines_per_cta(N);
+    const int G = blockDim.x / T;
     const int grp = threadIdx.x / T, lt = threadIdx.x % T;
     C* s = reinterpret_cast<C*>(smem_raw) + (size_t)grp * (N + (N >> 4));
     const int chan = blockIdx.x * G + grp;
@@ -535,8 +589,7 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
     }
     const bool even = (l & 1) == 0;
     const int line = live ? g.line0[gi] + (cplx ? 2 * local : local) : 0;
-    const R isc1 = (R)sqrt((double)N / 2.0), isc0 = (R)sqrt((double)N);
-    // unnormalised DCT-II coefficients X_k (pairs k = 2m, 2m+1); storage pair
+    // DCT-II coefficients X_k (pairs k = 2m, 2m+1); storage pair
     // (idx, idx+1) holds (k, k+1) for odd l and (k+1, k) for even l
     R re[8][2], im[8][2];
 #pragma unroll
@@ -561,9 +614,6 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
             X0.y = even ? im[u][1] : im[u][0];
             X1.x = even ? re[u][0] : re[u][1];
             X1.y = even ? im[u][0] : im[u][1];
-            const R s0 = (m == 0) ? isc0 : isc1;
-            X0.x *= s0; X0.y *= s0;
-            X1.x *= isc1; X1.y *= isc1;
             if (NS > 0) {
                 dst[u * st2] = X0;
                 dst[u * st2 + 1] = X1;
@@ -574,7 +624,8 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
         }
     }
     __syncthreads();
-    // V_k = conj(w_k) (X_k - i X_{N-k}); keep conj(V_k) for the IFFT-by-FFT
+    // V_k = conj(w_k) (X_k - i X_{N-k}), scaled with w_k (X_0 enters V_0 only);
+    // keep conj(V_k) for the IFFT-by-FFT
     C vk[16];
     const int st1 = pstride(T);
 #pragma unroll
@@ -586,7 +637,10 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
         C t;   // a - i b
         t.x = a.x + b.y;
         t.y = a.y - b.x;
-        const C v = cmulc(t, post[k]);
+        C w = post[k];
+        const R sc = (k == 0) ? dsc.c0 : dsc.c1;
+        w.x *= sc; w.y *= sc;
+        const C v = cmulc(t, w);
         vk[u].x = v.x;
         vk[u].y = -v.y;
     }
@@ -595,17 +649,16 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
     fft_from_registers<Q, NS>(s, vk, tw, sroot, N, lt, T);
     if (!live) return;
     const size_t ubase = g.uoff ? (size_t)g.uoff[chan] : (size_t)chan * N;   // caller's element offset
-    const R invN = (R)(1.0 / (double)N);
     const C* lo = s + padi(lt);
     const C* hi = s + padi(N - 1 - lt);
     const int st1b = pstride(T);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {   // j = lt + i T, N / 2 = 8 T
         const int j = lt + i * T;
-        C a = NS > 0 ? lo[i * st1b] : s[padi(j)];             // x_{2j} (conjugated, unscaled)
+        C a = NS > 0 ? lo[i * st1b] : s[padi(j)];             // x_{2j} (conjugated)
         C b = NS > 0 ? hi[-i * st1b] : s[padi(N - 1 - j)];    // x_{2j+1}
-        a.x *= invN; a.y = -a.y * invN;
-        b.x *= invN; b.y = -b.y * invN;
+        a.y = -a.y;
+        b.y = -b.y;
         if (even) { b.x = -b.x; b.y = -b.y; }
         if (cplx) {
             st_pair(reinterpret_cast<C*>(out) + ubase + 2 * j, a, b);
@@ -616,19 +669,25 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
     }
 }
 
+inline int nchannels(const GroupTable& g) { return g.chan0[g.ngroups]; }
+
 template <typename K>
-inline int launch_cfg(K kernel, int N, size_t elem, unsigned& threads, size_t& smem) {
-    const int G = lines_per_cta(N);
+inline int launch_cfg(K kernel, int N, int nchan, size_t elem, unsigned& blocks, unsigned& threads, size_t& smem) {
+    const int G = lines_per_cta(N, nchan);
+    blocks = (unsigned)((nchan + G - 1) / G);
     threads = (unsigned)(G * (N / 16));
     smem = (size_t)G * (N + N / 16) * elem;
     if (smem > 48 * 1024) return ensure_smem((const void*)kernel, smem);
     return DSBT_OK;
 }
 
-inline int nchannels(const GroupTable& g) { return g.chan0[g.ngroups]; }
-inline unsigned nblocks(const GroupTable& g, int N) {
-    const int G = lines_per_cta(N);
-    return (unsigned)((nchannels(g) + G - 1) / G);
+template <typename R>
+inline DctScale<R> fwd_scale(int N) {
+    return {(R)sqrt(1.0 / (double)N), (R)sqrt(2.0 / (double)N)};
+}
+template <typename R>
+inline DctScale<R> inv_scale(int N) {
+    return {(R)(1.0 / sqrt((double)N)), (R)(1.0 / sqrt(2.0 * (double)N))};
 }
 
 // Odd part Q of q = N / 256; every N = 256 q with q <= 32 has Q in 1..31.
@@ -642,8 +701,9 @@ inline int odd_part(int N) {
 
 template <typename R>
 using FwdKernel = void (*)(GroupTable, int, int, const R*, void*, void*, float*, const typename Cx<R>::T*,
-                           const typename Cx<R>::T*);
+                           const typename Cx<R>::T*, DctScale<R>);
 template <typename R>
-using InvKernel = void (*)(GroupTable, int, int, const R*, R*, const typename Cx<R>::T*, const typename Cx<R>::T*);
+using InvKernel = void (*)(GroupTable, int, int, const R*, R*, const typename Cx<R>::T*, const typename Cx<R>::T*,
+                           DctScale<R>);
 
 }  // namespace dsbt
