@@ -24,7 +24,10 @@
  *
  * Precision paths:
  *   - DSBT_F64 / DSBT_C128: everything in FP64 (sine/cosine transform by an
- *     FP64 FFT, T_l contraction by FP64 FMA).
+ *     FP64 FFT; T_l contraction to FP64 accuracy on the FP16 tensor cores, each
+ *     operand as 64 bits of fixed point relative to its line's largest magnitude
+ *     and multiplied exactly by base-256 digits; a line that holds an infinity or
+ *     a NaN gives NaNs).
  *   - DSBT_F32 / DSBT_C64: FP32 FFT, T_l contraction on the tcgen05 tensor
  *     cores as a compensated split product (T = T_hi + T_lo, x = x_hi + x_lo,
  *     T x ~ T_hi x_hi + T_hi x_lo + T_lo x_hi, FP32 accumulation in TMEM):

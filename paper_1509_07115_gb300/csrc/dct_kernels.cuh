@@ -685,9 +685,12 @@ template <typename R>
 inline DctScale<R> fwd_scale(int N) {
     return {(R)sqrt(1.0 / (double)N), (R)sqrt(2.0 / (double)N)};
 }
+// 1/sqrt(N), 1/sqrt(2N) as the reciprocals of the rounded forward factors times
+// N, so that a forward and an inverse transform scale by one as nearly as can be.
 template <typename R>
 inline DctScale<R> inv_scale(int N) {
-    return {(R)(1.0 / sqrt((double)N)), (R)(1.0 / sqrt(2.0 * (double)N))};
+    const DctScale<R> f = fwd_scale<R>(N);
+    return {(R)(1.0 / ((double)f.c0 * N)), (R)(1.0 / ((double)f.c1 * N))};
 }
 
 // Odd part Q of q = N / 256; every N = 256 q with q <= 32 has Q in 1..31.

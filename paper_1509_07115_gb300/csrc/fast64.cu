@@ -25,16 +25,15 @@
 // host by Arnoldi on the point grid with two Gram-Schmidt passes, so every
 // coefficient is a bounded projection (no monomial cancellation).
 //
-// On this part FP64 multiply-adds are the bound (a few per clock per SM), so
-// the kernels keep every lane on useful multiply-adds: lanes run over rows or
-// columns with the basis index k in the loop, and the few reductions across
-// lanes are shuffles over row chunks.
+// This file builds the operands (double); mm64.cu multiplies with them.
 #include <math.h>
 
 #include <algorithm>
 #include <thread>
+#include <utility>
 #include <vector>
 
+#include "mm64.cuh"
 #include "plan.cuh"
 
 namespace dsbt {
@@ -85,219 +84,6 @@ __global__ void k_fast_beta(const double* __restrict__ T64, const double* __rest
     beta[(((size_t)l * levels + j) * N + r) * KM + k] = s;
 }
 
-struct FastArgs {
-    const double* Q;       // all levels, [len_j][KM] at qoff[j]
-    const double* QT;      // all levels, [KM][len_j] at qoff[j]
-    const size_t* qoff;
-    const double* beta;    // [L][levels][N][KM]
-    const double* betaT;   // [L][levels][KM][N]
-    const double* nearT;   // [L][nleaf][FB][FB]: nearT[l][J][c][t] = T_l[J B + t][J B + c]
-    const double* T64;
-    int N, nleaf, levels, R;
-};
-
-__device__ __forceinline__ size_t mpos(const FastArgs& a, int j, int i, int line, int k) {
-    // scratch layout: level j block at sum_{j' < j} (nleaf >> j') R KM
-    size_t off = 0;
-    for (int q = 0; q < j; ++q) off += (size_t)(a.nleaf >> q) * a.R * KM;
-    return off + ((size_t)i * a.R + line) * KM + k;
-}
-
-// Groups are ordered by l, and the work of a block grows with l.  Projection
-// blocks take their group through this interleaving (0, n-1, 1, n-2, ...) so
-// that every run of consecutive blocks mixes light and heavy groups.
-__device__ __forceinline__ int interleave(int t, int n) { return (t & 1) ? n - 1 - (t >> 1) : (t >> 1); }
-
-constexpr int PROJ_THREADS = 256;
-
-// Interval i of level j is used when its right sibling exists (i even): the
-// rows of the sibling take it as a far interval.  Level j has nleaf >> (j+1)
-// used intervals, its rows are cut into nch_j <= 32 chunks, and a block takes
-// PROJ_THREADS / nch_j (line, k) pairs.  Blocks run over (level, tile, interval,
-// group), largest intervals first.
-__device__ __forceinline__ int proj_chunks(int j) { return min(32, 1 << j); }
-
-__device__ __forceinline__ bool proj_block(const FastArgs& a, int ngroups, int pmax, int b, int& j, int& gi,
-                                           int& i, int& tile) {
-    for (j = a.levels - 1; j >= 0; --j) {
-        const int used = a.nleaf >> (j + 1);
-        const int per = PROJ_THREADS / proj_chunks(j);
-        const int count = used * ngroups * ((pmax + per - 1) / per);
-        if (b < count) {
-            gi = interleave(b % ngroups, ngroups);
-            b /= ngroups;
-            i = 2 * (b % used);
-            tile = b / used;
-            return true;
-        }
-        b -= count;
-    }
-    return false;
-}
-
-// Projections onto the bases of the used intervals:
-//   forward (dir > 0): M_j[i][line][k] = sum_{t in I} Q_j[t][k] sqrt(w_t) f[line][t]
-//   inverse (dir < 0): W_j[i][line][k] = sum_{r in sibling} beta_{r,j}[k] b[line][r]
-// over the (line, k) pairs p = line K + k of a group (beta is zero on
-// completion rows, so those rows drop out).  Both operands are [row][KM].
-// Lane = (pair, chunk): a lane sums one chunk of len / nch rows, then the nch
-// lanes of a pair add their sums by shuffles.
-__global__ void __launch_bounds__(PROJ_THREADS) k_fast_project(FastArgs a, GroupTable g, int dir, int pmax,
-                                                               const double* __restrict__ in,
-                                                               double* __restrict__ out) {
-    int j, gi, i, tile;
-    if (!proj_block(a, g.ngroups, pmax, blockIdx.x, j, gi, i, tile)) return;
-    const int l = g.l[gi], K = l, line0 = g.line0[gi], nl = g.line0[gi + 1] - line0;
-    const int P = nl * K;
-    const int nch = proj_chunks(j), ppw = 32 / nch;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pw = (tile * (PROJ_THREADS / 32) + warp) * ppw;   // first pair of the warp
-    if (pw >= P) return;                                          // whole warp idle
-    const int q = lane & (nch - 1), pq = pw + lane / nch;
-    const int N = a.N, len = FB << j, clen = len / nch;
-    const int t0 = dir > 0 ? i * len : (i + 1) * len;
-    double acc = 0.0;
-    if (pq < P) {
-        const int line = pq / K, k = pq % K;
-        const double* x = in + (size_t)(line0 + line) * N + t0 + q * clen;
-        const double* o = (dir > 0 ? a.Q + a.qoff[j] : a.beta + (((size_t)l * a.levels + j) * N + t0) * KM) +
-                          (size_t)q * clen * KM + k;
-        const double x0 = (dir > 0 && t0 + q * clen == 0) ? sqrt_w(l, 0) * x[0] : x[0];
-        acc = o[0] * x0;
-#pragma unroll 8
-        for (int t = 1; t < clen; ++t) acc = fma(o[(size_t)t * KM], x[t], acc);
-    }
-    for (int s = nch >> 1; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-    if (q == 0 && pq < P) out[mpos(a, j, i, line0 + pq / K, pq % K)] = acc;
-}
-
-__device__ __forceinline__ void store_pair(double* out, size_t o0, int N, double s0, double s1, bool two,
-                                           const double2* phase, double2 ph) {
-    if (phase) {
-        out[o0] = s0 * ph.x - s1 * ph.y;
-        out[o0 + N] = s0 * ph.y + s1 * ph.x;
-    } else {
-        out[o0] = s0;
-        if (two) out[o0 + N] = s1;
-    }
-}
-
-// Forward output, lines in pairs (with a kinetic phase the pairs are the
-// (re, im) lines of a channel).  blockIdx.x < nleaf: leaf J, one thread per
-// regular row r = J B + t: near field sum_{c <= r in J} T_rc f_c from the
-// transposed leaf block, far field sum_j beta_{r,j} . M_j over the set bits j
-// of J.  blockIdx.x >= nleaf: completion rows, one warp per row (dense dot).
-__global__ void __launch_bounds__(FB) k_fast_eval(FastArgs a, GroupTable g, const double* __restrict__ in,
-                                                  const double* __restrict__ M, double* __restrict__ out,
-                                                  const double2* __restrict__ phase, int per_l) {
-    const int gi = gridDim.y - 1 - blockIdx.y, xb = blockIdx.x;   // largest l first
-    const int l = g.l[gi], K = l, line0 = g.line0[gi], nl = g.line0[gi + 1] - line0;
-    const int N = a.N, ne = n_extra(l);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (xb >= a.nleaf) {
-        const int r = (xb - a.nleaf) * (FB / 32) + w;
-        if (r >= ne) return;
-        const double* Trow = a.T64 + ((size_t)l * N + r) * N;
-        double2 ph = make_double2(1.0, 0.0);
-        if (phase) ph = per_l ? phase[(size_t)l * N + r] : phase[(size_t)(l & 1) * N + phase_entry(l, r, N)];
-        for (int line = 0; line < nl; line += 2) {
-            const bool two = line + 1 < nl;
-            const double* x0 = in + (size_t)(line0 + line) * N;
-            const double* x1 = two ? x0 + N : x0;
-            double s0 = 0.0, s1 = 0.0;
-            for (int c = lane; c < N; c += 32) {
-                const double t = Trow[c];
-                s0 = fma(t, x0[c], s0);
-                s1 = fma(t, x1[c], s1);
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            }
-            if (lane == 0) store_pair(out, (size_t)(line0 + line) * N + r, N, s0, s1, two, phase, ph);
-        }
-        return;
-    }
-    const int J = xb, r = J * FB + threadIdx.x;
-    if (J * FB + w * 32 + 31 < ne) return;   // the whole warp holds completion rows
-    const double* nt = a.nearT + (((size_t)l * a.nleaf + J) * FB) * FB + threadIdx.x;
-    const int cmax = (w + 1) * 32;           // T_rc = 0 for c > r
-    double2 ph = make_double2(1.0, 0.0);
-    if (phase) ph = per_l ? phase[(size_t)l * N + r] : phase[(size_t)(l & 1) * N + phase_entry(l, r, N)];
-    for (int line = 0; line < nl; line += 2) {
-        const bool two = line + 1 < nl;
-        const double* x0 = in + (size_t)(line0 + line) * N + J * FB;
-        const double* x1 = two ? x0 + N : x0;
-        double s0 = 0.0, s1 = 0.0;
-        for (int c = 0; c < cmax; ++c) {
-            const double t = nt[(size_t)c * FB];
-            s0 = fma(t, x0[c], s0);
-            s1 = fma(t, x1[c], s1);
-        }
-        for (int j = 0; j < a.levels; ++j) {
-            if (!((J >> j) & 1)) continue;
-            const int i = (J >> j) - 1;
-            const double* be = a.betaT + (((size_t)l * a.levels + j) * KM) * N + r;
-            const double* m0 = M + mpos(a, j, i, line0 + line, 0);
-            const double* m1 = two ? m0 + KM : m0;
-            for (int k = 0; k < K; ++k) {
-                const double b = be[(size_t)k * N];
-                s0 = fma(b, m0[k], s0);
-                s1 = fma(b, m1[k], s1);
-            }
-        }
-        if (r >= ne) store_pair(out, (size_t)(line0 + line) * N + r, N, s0, s1, two, phase, ph);
-    }
-}
-
-// Inverse output f = T^T b, one thread per column c of leaf J = blockIdx.x:
-// completion rows (dense), near field sum_{r >= c in J} T_rc b_r (T_rc = 0 for
-// r < c, so a warp starts at its first column), far field
-// sqrt(w_c) sum_j (Q_j W_j[i])_c over the levels j whose interval i holding c
-// is used.
-__global__ void __launch_bounds__(FB) k_fast_leaf_out(FastArgs a, GroupTable g, const double* __restrict__ in,
-                                                      const double* __restrict__ W, double* __restrict__ out) {
-    const int gi = gridDim.y - 1 - blockIdx.y, J = blockIdx.x;   // largest l first
-    const int l = g.l[gi], K = l, line0 = g.line0[gi], nl = g.line0[gi + 1] - line0;
-    const int N = a.N, ne = n_extra(l);
-    const int c = J * FB + threadIdx.x, w = threadIdx.x >> 5;
-    const double* T = a.T64 + (size_t)l * N * N + c;
-    const double sw = sqrt_w(l, c);
-    const int r_lo = max(ne, J * FB + w * 32), r_hi = (J + 1) * FB;
-    for (int line = 0; line < nl; line += 2) {
-        const bool two = line + 1 < nl;
-        const double* x0 = in + (size_t)(line0 + line) * N;
-        const double* x1 = two ? x0 + N : x0;
-        double s0 = 0.0, s1 = 0.0;
-        for (int r = 0; r < ne; ++r) {
-            const double t = T[(size_t)r * N];
-            s0 = fma(t, x0[r], s0);
-            s1 = fma(t, x1[r], s1);
-        }
-        for (int r = r_lo; r < r_hi; ++r) {
-            const double t = T[(size_t)r * N];
-            s0 = fma(t, x0[r], s0);
-            s1 = fma(t, x1[r], s1);
-        }
-        double f0 = 0.0, f1 = 0.0;
-        for (int j = 0; j < a.levels; ++j) {
-            const int i = J >> j;
-            if ((i & 1) || i + 1 >= (a.nleaf >> j)) continue;
-            const int len = FB << j;
-            const double* qt = a.QT + a.qoff[j] + (c - i * len);
-            const double* w0 = W + mpos(a, j, i, line0 + line, 0);
-            const double* w1 = two ? w0 + KM : w0;
-            for (int k = 0; k < K; ++k) {
-                const double q = qt[(size_t)k * len];
-                f0 = fma(q, w0[k], f0);
-                f1 = fma(q, w1[k], f1);
-            }
-        }
-        out[(size_t)(line0 + line) * N + c] = fma(sw, f0, s0);
-        if (two) out[(size_t)(line0 + line + 1) * N + c] = fma(sw, f1, s1);
-    }
-}
-
 // Build-time layouts: betaT[l][j][k][r] = beta[l][j][r][k] and the transposed
 // diagonal leaf blocks nearT[l][J][c][t] = T_l[J B + t][J B + c].
 __global__ void k_fast_transpose_beta(const double* __restrict__ beta, double* __restrict__ betaT, int N) {
@@ -306,10 +92,26 @@ __global__ void k_fast_transpose_beta(const double* __restrict__ beta, double* _
     betaT[(lj * KM + k) * N + r] = beta[(lj * N + r) * KM + k];
 }
 
-__global__ void k_fast_near(const double* __restrict__ T64, double* __restrict__ nearT, int N, int nleaf) {
+// near[l][J][t][c] the blocks themselves.
+__global__ void k_fast_near(const double* __restrict__ T64, double* __restrict__ near, double* __restrict__ nearT, int N,
+                            int nleaf) {
     const int J = blockIdx.x, l = blockIdx.y, c = threadIdx.x;
-    for (int t = 0; t < FB; ++t)
-        nearT[(((size_t)l * nleaf + J) * FB + c) * FB + t] = T64[((size_t)l * N + J * FB + t) * N + J * FB + c];
+    const size_t blk = ((size_t)l * nleaf + J) * FB * FB;
+    for (int t = 0; t < FB; ++t) {
+        const double v = T64[((size_t)l * N + J * FB + t) * N + J * FB + c];
+        nearT[blk + (size_t)c * FB + t] = v;
+        near[blk + (size_t)t * FB + c] = v;
+    }
+}
+
+// Doubles (|v| < 2) to the biased fixed-point words that the contraction takes
+// apart into digits (mm64.cuh), in place.
+__global__ void k_fast_fixed(double* p, size_t n) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint32_t lo, hi;
+    mm64::fixed_a(p[i], lo, hi);
+    reinterpret_cast<uint2*>(p)[i] = make_uint2(lo, hi);
 }
 
 }  // namespace
@@ -318,10 +120,14 @@ struct FastData {
     int nleaf = 0, levels = 0;
     double* Q = nullptr;
     double* QT = nullptr;
+    double* Qw = nullptr;    // [level][FB][KM]: the first leaf of Q_j with row 0 times sqrt(w_0) = 1/sqrt(2) (odd l)
+    double* QTw = nullptr;   // QT with column 0 of every level times sqrt(w_0) (odd l, intervals holding column 0)
     size_t* qoff = nullptr;
     double* beta = nullptr;
     double* betaT = nullptr;
+    double* near = nullptr;
     double* nearT = nullptr;
+    // every operand above holds biased fixed-point words once the plan is built
 };
 
 void poly_basis(int len, std::vector<double>& Q) { basis(len, Q); }
@@ -353,7 +159,7 @@ int fast_build(dsbt_plan* p, cudaStream_t st) {
         qoff[j] = qtot;
         qtot += Qh[j].size();
     }
-    std::vector<double> Qall(qtot), QTall(qtot);
+    std::vector<double> Qall(qtot), QTall(qtot), Qwall((size_t)levels * FB * KM), QTwall;
     for (int j = 0; j < levels; ++j) {
         const int len = FB << j;
         for (int t = 0; t < len; ++t)
@@ -362,16 +168,29 @@ int fast_build(dsbt_plan* p, cudaStream_t st) {
                 QTall[qoff[j] + (size_t)k * len + t] = Qh[j][(size_t)t * KM + k];
             }
     }
+    QTwall = QTall;
+    const double w0 = sqrt_w(1, 0);
+    for (int j = 0; j < levels; ++j)
+        for (int k = 0; k < KM; ++k) {
+            QTwall[qoff[j] + (size_t)k * (FB << j)] *= w0;
+            for (int t = 0; t < FB; ++t)
+                Qwall[((size_t)j * FB + t) * KM + k] = Qall[qoff[j] + (size_t)t * KM + k] * (t == 0 ? w0 : 1.0);
+        }
     const size_t L = (size_t)p->l_max + 1;
     const size_t nbeta = L * levels * N * KM;
     bool ok = cudaMalloc((void**)&f->Q, qtot * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&f->QT, qtot * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&f->Qw, Qwall.size() * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&f->QTw, qtot * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&f->qoff, levels * sizeof(size_t)) == cudaSuccess &&
               cudaMalloc((void**)&f->beta, nbeta * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&f->betaT, nbeta * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&f->near, L * N * FB * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&f->nearT, L * N * FB * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMemcpy(f->Q, Qall.data(), qtot * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(f->QT, QTall.data(), qtot * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaMemcpy(f->Qw, Qwall.data(), Qwall.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaMemcpy(f->QTw, QTwall.data(), qtot * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(f->qoff, qoff.data(), levels * sizeof(size_t), cudaMemcpyHostToDevice) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -380,7 +199,12 @@ int fast_build(dsbt_plan* p, cudaStream_t st) {
     }
     k_fast_beta<<<dim3(N, levels, (unsigned)L), KM, 0, st>>>(p->T64, f->Q, f->qoff, f->beta, N, levels);
     k_fast_transpose_beta<<<dim3(N, (unsigned)(L * levels)), KM, 0, st>>>(f->beta, f->betaT, N);
-    k_fast_near<<<dim3(f->nleaf, (unsigned)L), FB, 0, st>>>(p->T64, f->nearT, N, f->nleaf);
+    k_fast_near<<<dim3(f->nleaf, (unsigned)L), FB, 0, st>>>(p->T64, f->near, f->nearT, N, f->nleaf);
+    for (const auto& [ptr, n] : {std::make_pair(f->Q, qtot), std::make_pair(f->QT, qtot), std::make_pair(f->QTw, qtot),
+                                 std::make_pair(f->Qw, Qwall.size()), std::make_pair(f->beta, nbeta),
+                                 std::make_pair(f->betaT, nbeta), std::make_pair(f->near, L * N * FB),
+                                 std::make_pair(f->nearT, L * N * FB)})
+        k_fast_fixed<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ptr, n);
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -389,9 +213,12 @@ void fast_free(dsbt_plan* p) {
     if (!p || !p->fast) return;
     cudaFree(p->fast->Q);
     cudaFree(p->fast->QT);
+    cudaFree(p->fast->Qw);
+    cudaFree(p->fast->QTw);
     cudaFree(p->fast->qoff);
     cudaFree(p->fast->beta);
     cudaFree(p->fast->betaT);
+    cudaFree(p->fast->near);
     cudaFree(p->fast->nearT);
     delete p->fast;
     p->fast = nullptr;
@@ -404,33 +231,21 @@ size_t fast_scratch_bytes(const dsbt_plan* p, int lines) {
     return n * sizeof(double);
 }
 
-int contract_f64_fast(const dsbt_plan* p, const GroupTable& g, int dir, const double* in, double* out,
-                      const double2* phase, double* scratch, cudaStream_t st) {
+void fast_operands(const dsbt_plan* p, const double** Q, const double** QT, const double** Qw, const double** QTw,
+                   const size_t** qoff, const double** beta,
+                   const double** betaT, const double** near, const double** nearT, int* nleaf, int* levels) {
     const FastData* f = p->fast;
-    FastArgs a{f->Q, f->QT, f->qoff, f->beta, f->betaT, f->nearT, p->T64, p->N, f->nleaf, f->levels, g.total_lines};
-    const int per_l = p->knl != nullptr;
-    int pmax = 0, lmax = 0;
-    for (int gi = 0; gi < g.ngroups; ++gi) {
-        pmax = std::max(pmax, (g.line0[gi + 1] - g.line0[gi]) * g.l[gi]);
-        lmax = std::max(lmax, g.l[gi]);
-    }
-    ProfScope ps(kKContract64, st);
-    if (pmax > 0) {
-        long long blocks = 0;
-        for (int j = 0; j < f->levels; ++j) {
-            const int per = PROJ_THREADS / std::min(32, 1 << j);
-            blocks += (long long)(f->nleaf >> (j + 1)) * g.ngroups * ((pmax + per - 1) / per);
-        }
-        k_fast_project<<<(unsigned)blocks, PROJ_THREADS, 0, st>>>(a, g, dir, pmax, in, scratch);
-    }
-    if (dir > 0) {
-        const int ncomp = (n_extra(lmax) + FB / 32 - 1) / (FB / 32);
-        k_fast_eval<<<dim3(f->nleaf + ncomp, g.ngroups), FB, 0, st>>>(a, g, in, scratch, out, phase, per_l);
-    } else {
-        k_fast_leaf_out<<<dim3(f->nleaf, g.ngroups), FB, 0, st>>>(a, g, in, scratch, out);
-    }
-    DSBT_CUDA_TRY(cudaGetLastError());
-    return DSBT_OK;
+    *Q = f->Q;
+    *QT = f->QT;
+    *Qw = f->Qw;
+    *QTw = f->QTw;
+    *qoff = f->qoff;
+    *beta = f->beta;
+    *betaT = f->betaT;
+    *near = f->near;
+    *nearT = f->nearT;
+    *nleaf = f->nleaf;
+    *levels = f->levels;
 }
 
 }  // namespace dsbt

@@ -1,0 +1,116 @@
+// mm64.cuh -- FP64 products on the FP16 tensor cores through exact digits.
+//
+// The FP64 units of this part do 1.7 multiply-adds per clock and SM (measured;
+// 1.04 TFLOP/s over 152 SMs, the FP64 matrix instruction the same), the FP16
+// matrix instruction mma.sync m16n8k16 does 1024.  So an FP64 operand is
+// written as a fixed-point number of 64 bits relative to a power of two above
+// its largest magnitude, and that as eight balanced base-256 digits
+// D_0 .. D_7 in [-128, 127], each exact in FP16.  A product of two digits is at
+// most 2^14, so a sum of 2^10 of them is an integer of at most 2^24 and exact
+// in the FP32 accumulator (checked on the hardware for random and extreme
+// digits).  The 36 digit products D_i D_j with i + j <= 7 give
+//     sum_k a_k x_k = sum_s 2^(-8 s) sum_{i + j = s} sum_k D_i(a_k) D_j(x_k)
+// up to terms below 2^-64 of the operands' scales; the sums of each s are added
+// up as 64-bit integers and rounded to FP64 once.  FP64 arithmetic rounds every
+// multiply-add at 2^-53 of the partial sum instead; against 64-bit references
+// the results here are as close or closer (tests/test_mm64.py).  36 matrix
+// instructions of two clocks replace 2048 multiply-adds: 28 per clock and SM.
+//
+// K runs in blocks of 16.  Lane (g = lane / 4, t = lane % 4) of a warp holds
+// columns 4t .. 4t+3 of rows g and g + 8 of the A operand (one 32-byte piece of
+// each row), as the instruction's k indices 2t, 2t+1, 2t+8, 2t+9; the B operand
+// is read with the same permutation of k.
+#pragma once
+
+#include <stdint.h>
+
+#include <cuda_fp16.h>
+
+namespace dsbt {
+namespace mm64 {
+
+constexpr int ND = 8;                    // digits
+constexpr uint32_t kBias = 0x80808080u;  // every digit plus 128
+
+// 64-bit fixed point of v, m = v 2^(62 - E) truncated, plus the digit bias; shift
+// = 1 + (E's exponent field) - (v's), see exponent_of.
+__device__ __forceinline__ void fixed_point(uint32_t vl, uint32_t mh, int shift, int sign, uint32_t& lo, uint32_t& hi) {
+    const uint32_t s = min((uint32_t)shift, 63u);
+    unsigned long long m = ((unsigned long long)mh << 32 | (vl << 10)) >> s;
+    const unsigned long long sg = (unsigned long long)(long long)sign;   // 0 or all ones
+    m = (m ^ sg) + (((unsigned long long)kBias << 32 | kBias) - sg);
+    lo = (uint32_t)m;
+    hi = (uint32_t)(m >> 32);
+}
+
+// A operand: entries of orthogonal factors, |a| < 2, at the fixed scale 2^-61.
+__device__ __forceinline__ void fixed_a(double v, uint32_t& lo, uint32_t& hi) {
+    const uint32_t vl = (uint32_t)__double2loint(v), vh = (uint32_t)__double2hiint(v);
+    const uint32_t mh = (__funnelshift_l(vl, vh, 10) & 0x3fffffffu) | 0x40000000u;
+    fixed_point(vl, mh, 1024 - (int)((vh >> 20) & 0x7ffu), (int)vh >> 31, lo, hi);
+}
+
+// Exponent field of v (0 .. 2047); the largest over a line is its scale ef:
+// |v| < 2^(ef - 1022) = 2^E.
+__device__ __forceinline__ int exponent_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// B operand: v relative to its line's scale ef >= 64.  Zero and subnormals (field
+// 0) are shifted out.
+__device__ __forceinline__ void fixed_b(double v, int ef, uint32_t& lo, uint32_t& hi) {
+    const uint32_t vl = (uint32_t)__double2loint(v), vh = (uint32_t)__double2hiint(v);
+    const uint32_t mh = (__funnelshift_l(vl, vh, 10) & 0x3fffffffu) | 0x40000000u;
+    fixed_point(vl, mh, 1 + ef - (int)((vh >> 20) & 0x7ffu), (int)vh >> 31, lo, hi);
+}
+
+// The same for any scale: a line whose largest magnitude is below 2^-958.
+static __device__ __noinline__ void fixed_b_tiny(double v, int ef, uint32_t& lo, uint32_t& hi) {
+    const uint32_t vl = (uint32_t)__double2loint(v), vh = (uint32_t)__double2hiint(v);
+    const int e = (int)((vh >> 20) & 0x7ffu);
+    const uint32_t mh = (__funnelshift_l(vl, vh, 10) & 0x3fffffffu) | (e ? 0x40000000u : 0u);
+    fixed_point(vl, mh, 1 + max(ef, 1) - max(e, 1), (int)vh >> 31, lo, hi);
+}
+
+// Digit d of two fixed-point words as a pair of FP16 integers: byte b becomes
+// 1024 + b (0x6400 | b), minus 1152.
+template <int d>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t lo0, uint32_t hi0, uint32_t lo1, uint32_t hi1) {
+    constexpr uint32_t b = 3 - (d & 3);
+    const uint32_t p = d < 4 ? __byte_perm(hi0, hi1, b | ((4 + b) << 8)) : __byte_perm(lo0, lo1, b | ((4 + b) << 8));
+    const uint32_t q = (p & 0x00ff00ffu) | 0x64006400u;
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&q), __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480)));
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// The eight digits of a thread's four consecutive k of one row: [d][pair].
+struct Digits4 {
+    uint32_t d[ND][2];
+    __device__ __forceinline__ void set(const uint32_t* lo, const uint32_t* hi) {
+#define DSBT_DIGIT(k)                                              \
+    d[k][0] = digit_pair<k>(lo[0], hi[0], lo[1], hi[1]);           \
+    d[k][1] = digit_pair<k>(lo[2], hi[2], lo[3], hi[3]);
+        DSBT_DIGIT(0) DSBT_DIGIT(1) DSBT_DIGIT(2) DSBT_DIGIT(3) DSBT_DIGIT(4) DSBT_DIGIT(5) DSBT_DIGIT(6) DSBT_DIGIT(7)
+#undef DSBT_DIGIT
+    }
+};
+
+__device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// A result: sum = 2^(E - 67) (hi 2^32 + lo).  |sum| <= ||a|| ||x|| < 2^(E + 6.5)
+// for K <= 8192, so hi 2^20 stays below 2^62 and one 64-bit integer with the
+// unit 2^(E - 55) holds it.
+__device__ __forceinline__ double to_double(long long hi, long long lo, int ef) {
+    if (ef == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);   // a line with an infinity or NaN
+    const long long v = hi * (1ll << 20) + ((lo + 2048) >> 12);
+    const int e = max(ef, 1) - 1022 - 55;
+    const double s = e > -1022 ? __hiloint2double((e + 1023) << 20, 0) : ldexp(1.0, e);
+    return (double)v * s;
+}
+
+}  // namespace mm64
+}  // namespace dsbt

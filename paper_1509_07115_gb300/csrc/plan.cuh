@@ -122,7 +122,7 @@ int dct_inverse_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const do
 int dct_inverse_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const float* in,
                     float* out, cudaStream_t st);
 
-// ---- FP64 contraction (gemm_f64.cu)
+// ---- FP64 contraction (mm64.cu)
 // in_cplx / out_cplx = 1: the caller's interleaved complex layout (line 2j+s of a
 // group is part s of its channel j); 0: planar lines [line][N].
 // dir = +1: out = T_l in (forward), dir = -1: out = T_l^T in (inverse).
@@ -131,13 +131,19 @@ int dct_inverse_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
 int contract_f64(const dsbt_plan* p, const GroupTable& g, int dir, const double* in, int in_cplx,
                  double* out, int out_cplx, const double2* phase, cudaStream_t st,
                  double* fast_scratch = nullptr);
-// DSBT_PLAN_FAST64 (fast64.cu)
+// DSBT_PLAN_FAST64 (fast64.cu); fast_scratch: its moments, fast_scratch_bytes of
+// the call's lines, or nullptr for the dense factors
 bool fast_supported(int N);
 int fast_build(dsbt_plan* p, cudaStream_t st);
 void fast_free(dsbt_plan* p);
 size_t fast_scratch_bytes(const dsbt_plan* p, int lines);
-int contract_f64_fast(const dsbt_plan* p, const GroupTable& g, int dir, const double* in, double* out,
-                      const double2* phase, double* scratch, cudaStream_t st);
+// Device operands of the interval scheme: bases [len_j][64] and transposes at
+// qoff[j] (Qw, QTw: with the weight of column 0 for odd l), projections
+// beta [l][j][r][64] and [l][j][64][r], leaf blocks and transposes, all as
+// biased fixed-point words (mm64.cuh).
+void fast_operands(const dsbt_plan* p, const double** Q, const double** QT, const double** Qw, const double** QTw,
+                   const size_t** qoff, const double** beta,
+                   const double** betaT, const double** near, const double** nearT, int* nleaf, int* levels);
 // Orthonormal basis [len][64] of the polynomials of degree < min(64, len) on
 // the points x_t = (2t+1)/len - 1 (Arnoldi with two Gram-Schmidt passes).
 void poly_basis(int len, std::vector<double>& Q);
