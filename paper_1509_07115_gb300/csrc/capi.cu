@@ -294,20 +294,24 @@ int run_inverse(const dsbt_plan* p, const GroupTable& g, int dtype, const void* 
     return dct_inverse_f32(p, g, cplx, w.planar, (float*)out, st);
 }
 
+int fill_phase64(const dsbt_plan* p, const Workspace& w, double tau, cudaStream_t st) {
+    ProfScope ps(kKPhase, st);
+    const int rows = phase_rows(p);
+    k_phase<<<(rows * p->N + 255) / 256, 256, 0, st>>>(w.ph64, nullptr, p->N, p->dk, tau, p->knl, rows);
+    DSBT_CUDA_TRY(cudaGetLastError());
+    return DSBT_OK;
+}
+
+// phase_ready (FP64): the workspace's table is already that of tau.
 int run_kinetic(const dsbt_plan* p, const GroupTable& g, int dtype, double tau, const void* in, void* out,
-                void* ws, cudaStream_t st) {
+                void* ws, cudaStream_t st, bool phase_ready = false) {
     if (g.total_lines == 0) return DSBT_OK;
     Workspace w = carve(p, ws, g.chan0[g.ngroups], dtype);
     const int N = p->N;
     int rc;
     if (is_fp64(dtype)) {
-        {
-            ProfScope ps(kKPhase, st);
-            const int rows = phase_rows(p);
-            k_phase<<<(rows * N + 255) / 256, 256, 0, st>>>(w.ph64, nullptr, N, p->dk, tau, p->knl, rows);
-        }
-        DSBT_CUDA_TRY(cudaGetLastError());
-        rc = dct_forward_f64(p, g, true, (const double*)in, w.f64a, st);
+        rc = phase_ready ? DSBT_OK : fill_phase64(p, w, tau, st);
+        if (!rc) rc = dct_forward_f64(p, g, true, (const double*)in, w.f64a, st);
         if (!rc) rc = contract_f64(p, g, +1, w.f64a, 0, w.f64b, 0, w.ph64, st, w.fast);
         if (!rc) rc = contract_f64(p, g, -1, w.f64b, 0, w.f64a, 0, nullptr, st, w.fast);
         if (!rc) rc = dct_inverse_f64(p, g, true, w.f64a, (double*)out, st);
@@ -364,7 +368,7 @@ int grouped_call(int which, const dsbt_plan* p, const int* counts, int dtype, do
     if (which == 1) return run_inverse(p, g, dtype, in, out, ws, st);
     DSBT_CHECK_ARG(is_complex(dtype), "kinetic step needs a complex dtype");
     DSBT_CHECK_ARG(isfinite(tau), "tau must be finite");
-    return run_kinetic(p, g, dtype, tau, in, out, ws, st);
+    return run_kinetic(p, g, dtype, tau, in, out, ws, st, which == kKineticReady && is_fp64(dtype));
 }
 
 int single_call(int which, const dsbt_plan* p, int l, int nchan, int dtype, const void* in, void* out,
@@ -395,6 +399,14 @@ int forward_grouped_with_scratch(const dsbt_plan* p, const int* counts, int dtyp
 int grouped_device_call(int which, const dsbt_plan* p, const int* counts, int dtype, double tau,
                         const void* in, void* out, void* ws, size_t ws_b, cudaStream_t st, const long long* uoff) {
     return grouped_call(which, p, counts, dtype, tau, in, out, ws, ws_b, st, uoff);
+}
+
+int kinetic_phase_fill(const dsbt_plan* p, void* ws, int total_channels, double tau, cudaStream_t st) {
+    return fill_phase64(p, carve(p, ws, total_channels, DSBT_C128), tau, st);
+}
+
+const double2* kinetic_phase_table(const dsbt_plan* p, void* ws, int total_channels) {
+    return carve(p, ws, total_channels, DSBT_C128).ph64;
 }
 
 // Grouped kinetic step with a scratch buffer supplied by the caller of this

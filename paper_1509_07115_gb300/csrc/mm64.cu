@@ -299,15 +299,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
             }
         } else {
 #pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int s = 0; s < ND; ++s)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const long long v = __float2int_rn(acc[n * ND + s][c]);
-                        if (s < 4) shi[n * 4 + c] += v * (1ll << (8 * (3 - s)));
-                        else slo[n * 4 + c] += v * (1ll << (8 * (7 - s)));
-                    }
+            for (int n = 0; n < NT; ++n) drain8(acc + n * ND, shi + n * 4, slo + n * 4);
         }
     };
 
@@ -367,26 +359,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     for (int r0 = 0; r0 < K; r0 += KR) {
         const int kr = min(KR, K - r0);
         const bool on = tk < kr;
-        // digits of one task's columns to shared memory
-        auto put_digits = [&](int j, int e, const double* v) {
-            uint32_t wl[4], wh[4];
-            if (e >= 64) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) fixed_b(v[c], e, wl[c], wh[c]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) fixed_b_tiny(v[c], e, wl[c], wh[c]);
-            }
-            Digits4 d;
-            d.set(wl, wh);
-            __half* dst = dig + (size_t)j * BS + tk;
-#pragma unroll
-            for (int q = 0; q < ND; ++q)
-                *reinterpret_cast<uint2*>(dst + (size_t)q * NL * BS) = make_uint2(d.d[q][0], d.d[q][1]);
-        };
-        auto exponent4 = [](const double* v) {
-            return max(max(exponent_of(v[0]), exponent_of(v[1])), max(exponent_of(v[2]), exponent_of(v[3])));
-        };
+        auto put_digits = [&](int j, int e, const double* v) { put_digits4(dig + (size_t)j * BS + tk, NL * BS, v, e); };
         const double* p = nullptr;
         int step = 0, pair = 0, odd = 0;
         if (on) {

@@ -22,6 +22,7 @@
 // is read with the same permutation of k.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 
 #include <cuda_fp16.h>
@@ -48,6 +49,13 @@ __device__ __forceinline__ void fixed_a(double v, uint32_t& lo, uint32_t& hi) {
     const uint32_t vl = (uint32_t)__double2loint(v), vh = (uint32_t)__double2hiint(v);
     const uint32_t mh = (__funnelshift_l(vl, vh, 10) & 0x3fffffffu) | 0x40000000u;
     fixed_point(vl, mh, 1024 - (int)((vh >> 20) & 0x7ffu), (int)vh >> 31, lo, hi);
+}
+
+// The words of fixed_a for a small host table.
+inline uint2 fixed_a_host(double v) {
+    const long long m = (long long)ldexp(v, 61);   // |v| < 2; truncates toward zero as the device does
+    const unsigned long long b = (unsigned long long)m + ((unsigned long long)kBias << 32 | kBias);
+    return make_uint2((uint32_t)b, (uint32_t)(b >> 32));
 }
 
 // Exponent field of v (0 .. 2047); the largest over a line is its scale ef:
@@ -99,6 +107,91 @@ __device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uin
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// FP32 sums of the digit products of one n8 tile, by i + j, added to 64-bit sums:
+// hi takes i + j <= 3 in units of 2^24, lo the rest.
+__device__ __forceinline__ void drain8(const float (*acc)[4], long long* hi, long long* lo) {
+#pragma unroll
+    for (int s = 0; s < ND; ++s)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const long long v = __float2int_rn(acc[s][c]);
+            if (s < 4) hi[c] += v * (1ll << (8 * (3 - s)));
+            else lo[c] += v * (1ll << (8 * (7 - s)));
+        }
+}
+
+// All 36 digit products of one unit (16 rows x 16 k) with one n8 tile.  b: the
+// thread's columns (lane row g of digit 0); rows of one digit are dstride halfs apart.
+__device__ __forceinline__ void unit8(float (*acc)[4], const Digits4& d0, const Digits4& d1, const __half* b, int dstride) {
+#pragma unroll
+    for (int j = 0; j < ND; ++j) {
+        const uint2 v = *reinterpret_cast<const uint2*>(b + (size_t)j * dstride);
+#pragma unroll
+        for (int i = 0; i + j < ND; ++i)
+            mma16816(acc[i + j], d0.d[i][0], d1.d[i][0], d0.d[i][1], d1.d[i][1], v.x, v.y);
+    }
+}
+
+// Product of a 16-row block of fixed-point words (row stride lda, K = 16 units) with
+// NT n8 tiles of digits [ND][8 NT][bs] in shared memory; K at most 128.  Results:
+// hi, lo[n][c] with c = 0, 1: row g, columns 2t, 2t + 1 of tile n; c = 2, 3: row g + 8.
+template <int NT>
+__device__ __forceinline__ void block_product(const uint2* A, int lda, int units, const __half* dig, int bs, int lane,
+                                              long long (*hi)[4], long long (*lo)[4]) {
+    const int g = lane >> 2, t = lane & 3;
+    float acc[NT][ND][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int s = 0; s < ND; ++s)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[n][s][c] = 0.f;
+    const uint4* r0 = reinterpret_cast<const uint4*>(A + (size_t)g * lda + 4 * t);
+    const uint4* r1 = reinterpret_cast<const uint4*>(A + (size_t)(g + 8) * lda + 4 * t);
+    uint4 w[4] = {__ldg(r0), __ldg(r0 + 1), __ldg(r1), __ldg(r1 + 1)};
+    for (int u = 0; u < units; ++u) {
+        uint32_t l0[4] = {w[0].x, w[0].z, w[1].x, w[1].z}, h0[4] = {w[0].y, w[0].w, w[1].y, w[1].w};
+        uint32_t l1[4] = {w[2].x, w[2].z, w[3].x, w[3].z}, h1[4] = {w[2].y, w[2].w, w[3].y, w[3].w};
+        if (u + 1 < units) {
+            r0 += 8;
+            r1 += 8;
+            w[0] = __ldg(r0); w[1] = __ldg(r0 + 1); w[2] = __ldg(r1); w[3] = __ldg(r1 + 1);
+        }
+        Digits4 d0, d1;
+        d0.set(l0, h0);
+        d1.set(l1, h1);
+#pragma unroll
+        for (int n = 0; n < NT; ++n) unit8(acc[n], d0, d1, dig + (size_t)(n * 8 + g) * bs + u * 16 + 4 * t, 8 * NT * bs);
+    }
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) hi[n][c] = lo[n][c] = 0;
+        drain8(acc[n], hi[n], lo[n]);
+    }
+}
+
+// Digits of four consecutive k of one column to its place in [ND][ncols][bs] (dst:
+// the column's first of the four, digit 0).
+__device__ __forceinline__ void put_digits4(__half* dst, int dstride, const double* v, int ef) {
+    uint32_t wl[4], wh[4];
+    if (ef >= 64) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) fixed_b(v[c], ef, wl[c], wh[c]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) fixed_b_tiny(v[c], ef, wl[c], wh[c]);
+    }
+    Digits4 d;
+    d.set(wl, wh);
+#pragma unroll
+    for (int q = 0; q < ND; ++q) *reinterpret_cast<uint2*>(dst + (size_t)q * dstride) = make_uint2(d.d[q][0], d.d[q][1]);
+}
+
+__device__ __forceinline__ int exponent4(const double* v) {
+    return max(max(exponent_of(v[0]), exponent_of(v[1])), max(exponent_of(v[2]), exponent_of(v[3])));
 }
 
 // A result: sum = 2^(E - 67) (hi 2^32 + lo).  |sum| <= ||a|| ||x|| < 2^(E + 6.5)

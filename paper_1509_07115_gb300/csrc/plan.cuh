@@ -84,6 +84,13 @@ int grouped_device_call(int which, const dsbt_plan* p, const int* counts, int dt
                         const void* in, void* out, void* ws, size_t ws_b, cudaStream_t st,
                         const long long* uoff = nullptr);
 
+// which = kKineticReady: the kinetic step (FP64, complex) with the phase table that
+// kinetic_phase_fill put into the workspace (of `total_channels` complex128
+// channels); forward, inverse and such kinetic calls leave the table alone.
+enum : int { kKineticReady = 3 };
+int kinetic_phase_fill(const dsbt_plan* p, void* ws, int total_channels, double tau, cudaStream_t st);
+const double2* kinetic_phase_table(const dsbt_plan* p, void* ws, int total_channels);
+
 // ---- plan build (plan.cu)
 int plan_build_factors(dsbt_plan* p, cudaStream_t st);
 int plan_probe(dsbt_plan* p, cudaStream_t st);

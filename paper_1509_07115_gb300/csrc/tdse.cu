@@ -12,20 +12,28 @@
 // Pbar_l(eta_j) sqrt(w_j) the orthonormal angular transform of Sec. 4.1
 // (associated Legendre functions for m = 0), V(r) = -Z / sqrt(r^2 + a2).
 //
+// Adjacent half steps share the angular grid and P is orthogonal, so Q_{s+1} Q_s =
+// P diag_j exp(-i [2 V(r_i) + (E_s + E_{s+1}) r_i eta_j] tau/2) P^T is one pass: a
+// propagation alternates Kin with such merged passes and has single ones at its
+// ends only.
+//
 // Adjoint: every factor is unitary and B, P are real orthogonal (Eq. (25),
 // T^{-1} = T^T), so U_s^H = Q_s^H Kin^H Q_s^H is the same step with tau -> -tau.
 // For the observable O = sum_{r_i > r_cut} |psi_S|^2 and lambda_S = Pi psi_S:
-//     mu = Q_s^H lambda_{s+1},  nu = Kin^H mu,  lambda_s = Q_s^H nu,
-//     dO/dE_s = tau Im( <lambda_{s+1}, R psi_{s+1}> + <nu, R a_s> ),  a_s = Q_s psi_s,
+//     nu_s = Kin^H Q_s^H lambda_{s+1},  lambda_s = Q_s^H nu_s,
+//     dO/dE_s = tau Im( <lambda_{s+1}, R psi_{s+1}> + <nu_s, R a_s> ),  a_s = Q_s psi_s,
 // where R = diag(r_i eta_j) on the angular grid (the field coupling r cos(theta)).
-// The inner products are accumulated inside the potential kernel from the
-// angular-grid values it already holds.
+// R commutes with Q_s, so <nu_s, R a_s> = <lambda_s, R psi_s> = g_s and
+//     dO/dE_s = tau (Im g_s + Im g_{s+1}),   g_S real (lambda_S = Pi psi_S),
+// with g_s = <P^T nu_s, R P^T a_s> from grid values that the merged passes hold:
+// the forward pass of a segment stores P^T a_s, the adjoint pass meets P^T nu_s.
 #include <math.h>
 
 #include <new>
 #include <algorithm>
 #include <vector>
 
+#include "mm64.cuh"
 #include "plan.cuh"
 
 namespace dsbt {
@@ -42,6 +50,7 @@ struct dsbt_tdse {
     int m0;         // |m|: channels are l = m0 .. m0 + L - 1
     double dr, tau, Z, a2;
     double* P;      // [L][L] angular transform
+    uint2* Pw;      // its fixed-point words (mm64.cuh): [64][64] P^T by node pairs, then [64][64] P
     double* V;      // [N] potential
     double* rr;     // [N] radii
     double* eta;    // [L] nodes
@@ -52,8 +61,9 @@ namespace dsbt {
 
 namespace {
 
-constexpr int TI = 16;          // radial points per tile of the angular kernel
+constexpr int TI = 8;           // radial points per tile of the angular kernels: 16 real columns
 constexpr int kLMax = 64;
+constexpr int AB = kLMax + 16;  // halfs per digit row of a tile (mm64.cuh)
 
 // Gauss-Legendre nodes and weights by Newton's method on P_L (three-term
 // recurrence for P_L and its derivative).
@@ -158,80 +168,131 @@ __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// y = P diag(exp(-i [V + E r eta] ht)) P^T x on a tile of TI radial points
-// (ht = +tau/2 forward, -tau/2 adjoint).  With aux != nullptr, also adds
-// gscale * Im( sum conj(x_eta) r eta aux_eta ) into *gacc.  x and y may alias.
-__global__ void __launch_bounds__(256) k_tdse_potential(const double2* __restrict__ x, double2* y,
-                                                        const double* __restrict__ P,
-                                                        const double* __restrict__ V,
-                                                        const double* __restrict__ rr,
-                                                        const double* __restrict__ eta, int L, int N,
-                                                        const double* __restrict__ E, int eidx, double ht,
-                                                        const double2* __restrict__ aux, double gscale,
-                                                        double* gacc) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    double* Ps = reinterpret_cast<double*>(sm);                    // [L][L]
-    double2* xs = reinterpret_cast<double2*>(Ps + kLMax * kLMax);  // [L][TI]
-    double2* xe = xs + kLMax * TI;                                 // [L][TI]
-    double2* as = xe + kLMax * TI;                                 // [L][TI]
-    __shared__ double red[2][8];
-    const int i0 = blockIdx.x * TI;
-    const int tid = threadIdx.x;
-    for (int k = tid; k < L * L; k += blockDim.x) Ps[k] = P[k];
-    for (int k = tid; k < L * TI; k += blockDim.x) {
-        const int l = k / TI, t = k % TI;
-        const int i = i0 + t;
-        xs[k] = (i < N) ? x[(size_t)l * N + i] : make_double2(0.0, 0.0);
-        if (aux) as[k] = (i < N) ? aux[(size_t)l * N + i] : make_double2(0.0, 0.0);
+// The angular kernels take TI radial points (16 real columns) through P^T, a
+// diagonal and P.  Both products run on the tensor cores through exact digits
+// (mm64.cuh): as FP64 multiply-adds they took 80 us per pass at L = 64, N = 2048,
+// the FP64 pipe's whole rate.  What is left on that pipe are the phases, so the
+// nodes go in pairs: row g of a 16-row block is node j = 8 m + g and row g + 8 its
+// mirror L - 1 - j (eta_{L-1-j} = -eta_j), both in one thread, and one sine and
+// cosine serve both.
+struct AngularShared {
+    __half dig[mm64::ND][2 * TI][AB];
+    double2 grid[kLMax][TI];
+    int ef[2][2 * TI];
+    double2 vph[TI];
+};
+
+// Digits of v[c] = rows 4 kq + c of column pair t (re, im); every thread of the CTA.
+__device__ __forceinline__ void angular_digits(AngularShared& sh, int pass, int kq, int t, const double2* v) {
+    const double re[4] = {v[0].x, v[1].x, v[2].x, v[3].x}, im[4] = {v[0].y, v[1].y, v[2].y, v[3].y};
+    int er = mm64::exponent4(re), ei = mm64::exponent4(im);
+#pragma unroll
+    for (int o = TI; o < 32; o <<= 1) {   // lanes of one point
+        er = max(er, __shfl_xor_sync(0xffffffffu, er, o));
+        ei = max(ei, __shfl_xor_sync(0xffffffffu, ei, o));
+    }
+    if ((threadIdx.x & 31) < TI) {
+        atomicMax(&sh.ef[pass][2 * t], er);
+        atomicMax(&sh.ef[pass][2 * t + 1], ei);
     }
     __syncthreads();
-    const double Ev = E ? E[eidx] : 0.0;
+    mm64::put_digits4(&sh.dig[0][2 * t][4 * kq], 2 * TI * AB, re, sh.ef[pass][2 * t]);
+    mm64::put_digits4(&sh.dig[0][2 * t + 1][4 * kq], 2 * TI * AB, im, sh.ef[pass][2 * t + 1]);
+    __syncthreads();
+}
+
+// y = P diag(exp(-i [w V + (E_e1 + E_e2) r eta] ht)) P^T x (w = 2, or w = 1 and no
+// second sample for e2 < 0; ht = +tau/2 forward, -tau/2 adjoint).  x and y may
+// alias; y may be null (no way back).  grid_out: also stores the grid values
+// [L][N] after the phase.  grid_in: adds gscale * sum Im(conj(P^T x) r eta grid_in)
+// into *g1 and, unless null, *g2.
+__global__ void __launch_bounds__(128) k_tdse_potential(const double2* x, double2* y, const uint2* __restrict__ Pw,
+                                                        const double* __restrict__ V, const double* __restrict__ rr,
+                                                        const double* __restrict__ eta, int L, int N,
+                                                        const double* __restrict__ E, int e1, int e2, double ht,
+                                                        double2* grid_out, const double2* __restrict__ grid_in,
+                                                        double gscale, double* g1, double* g2) {
+    __shared__ AngularShared sh;
+    __shared__ double red[4];
+    const int i0 = blockIdx.x * TI, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int t = tid % TI, kq = tid / TI, i = i0 + t;   // N is a multiple of 256
+    const int L16 = (L + 15) & ~15, half = (L + 1) / 2;
+    double2 v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = 4 * kq + c < L ? x[(size_t)(4 * kq + c) * N + i] : make_double2(0.0, 0.0);
+    if (tid < 4 * TI) sh.ef[tid / (2 * TI)][tid % (2 * TI)] = 0;
+    if (tid < TI) {
+        double sn, cs;
+        sincos(-(e2 >= 0 ? 2.0 : 1.0) * V[i] * ht, &sn, &cs);
+        sh.vph[t] = make_double2(cs, sn);
+    }
+    for (int k = tid; k < (L16 - L) * TI; k += blockDim.x) sh.grid[L + k / TI][k % TI] = make_double2(0.0, 0.0);
+    __syncthreads();
+    angular_digits(sh, 0, kq, t, v);
+    const double Ev = (E ? E[e1] : 0.0) + (E && e2 >= 0 ? E[e2] : 0.0);
     double gim = 0.0;
-    for (int k = tid; k < L * TI; k += blockDim.x) {   // to the angular grid
-        const int j = k / TI, t = k % TI;
-        double2 s = make_double2(0.0, 0.0), sa = make_double2(0.0, 0.0);
-        for (int l = 0; l < L; ++l) {
-            const double pj = Ps[l * L + j];
-            const double2 v = xs[l * TI + t];
-            s.x = fma(pj, v.x, s.x);
-            s.y = fma(pj, v.y, s.y);
-            if (aux) {
-                const double2 va = as[l * TI + t];
-                sa.x = fma(pj, va.x, sa.x);
-                sa.y = fma(pj, va.y, sa.y);
+    if (8 * warp < half) {   // to the angular grid
+        long long hi[2][4], lo[2][4];
+        mm64::block_product<2>(Pw + (size_t)warp * 16 * kLMax, kLMax, L16 / 16, &sh.dig[0][0][0], AB, lane, hi, lo);
+        const int g = lane >> 2, tq = lane & 3, j = 8 * warp + g, jm = L - 1 - j;
+        if (j < half) {
+            const double ej = eta[j];
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const int tp = 4 * n + tq, ip = i0 + tp, er = sh.ef[0][2 * tp], ei = sh.ef[0][2 * tp + 1];
+                const double re = rr[ip] * ej;
+                double2 a = make_double2(mm64::to_double(hi[n][0], lo[n][0], er), mm64::to_double(hi[n][1], lo[n][1], ei));
+                double2 b = make_double2(mm64::to_double(hi[n][2], lo[n][2], er), mm64::to_double(hi[n][3], lo[n][3], ei));
+                if (grid_in) {   // the middle node of an odd L is its own mirror
+                    const double2 ga = grid_in[(size_t)j * N + ip];
+                    gim += re * (a.x * ga.y - a.y * ga.x);
+                    if (jm != j) {
+                        const double2 gb = grid_in[(size_t)jm * N + ip];
+                        gim -= re * (b.x * gb.y - b.y * gb.x);
+                    }
+                }
+                double sn, cs;
+                sincos(-Ev * re * ht, &sn, &cs);
+                const double2 w = sh.vph[tp];
+                a = cmul2(cmul2(a, w), make_double2(cs, sn));
+                b = cmul2(cmul2(b, w), make_double2(cs, -sn));
+                sh.grid[j][tp] = a;
+                if (grid_out) grid_out[(size_t)j * N + ip] = a;
+                if (jm != j) {
+                    sh.grid[jm][tp] = b;
+                    if (grid_out) grid_out[(size_t)jm * N + ip] = b;
+                }
             }
         }
-        const int i = i0 + t;
-        if (i < N) {
-            const double r = rr[i];
-            if (aux) gim += r * eta[j] * (s.x * sa.y - s.y * sa.x);   // Im(conj(s) sa) r eta
-            double sn, cs;
-            sincos(-(V[i] + Ev * r * eta[j]) * ht, &sn, &cs);
-            s = cmul2(s, make_double2(cs, sn));
-        }
-        xe[k] = s;
+    }
+    if (grid_in) {
+        for (int o = 16; o > 0; o >>= 1) gim += __shfl_xor_sync(0xffffffffu, gim, o);
+        if (lane == 0) red[warp] = gim;
     }
     __syncthreads();
-    for (int k = tid; k < L * TI; k += blockDim.x) {   // back to l
-        const int l = k / TI, t = k % TI;
-        double2 s = make_double2(0.0, 0.0);
-        for (int j = 0; j < L; ++j) {
-            const double pl = Ps[l * L + j];
-            const double2 v = xe[j * TI + t];
-            s.x = fma(pl, v.x, s.x);
-            s.y = fma(pl, v.y, s.y);
-        }
-        const int i = i0 + t;
-        if (i < N) y[(size_t)l * N + i] = s;
+    if (grid_in && tid == 0) {
+        const double sum = gscale * (red[0] + red[1] + red[2] + red[3]);
+        atomicAdd(g1, sum);
+        if (g2) atomicAdd(g2, sum);
     }
-    if (aux) {
-        for (int o = 16; o > 0; o >>= 1) gim += __shfl_xor_sync(0xffffffffu, gim, o);
-        if ((tid & 31) == 0) red[0][tid >> 5] = gim;
-        __syncthreads();
-        if (tid == 0) {
-            double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[0][w];
-            atomicAdd(gacc, gscale * t);
+    if (!y) return;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = 4 * kq + c < L16 ? sh.grid[4 * kq + c][t] : make_double2(0.0, 0.0);
+    angular_digits(sh, 1, kq, t, v);
+    if (16 * warp < L) {   // back to l
+        long long hi[2][4], lo[2][4];
+        mm64::block_product<2>(Pw + (size_t)(kLMax + warp * 16) * kLMax, kLMax, L16 / 16, &sh.dig[0][0][0], AB, lane, hi,
+                               lo);
+        const int l = 16 * warp + (lane >> 2);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const int tp = 4 * n + (lane & 3), er = sh.ef[1][2 * tp], ei = sh.ef[1][2 * tp + 1];
+            if (l < L)
+                y[(size_t)l * N + i0 + tp] =
+                    make_double2(mm64::to_double(hi[n][0], lo[n][0], er), mm64::to_double(hi[n][1], lo[n][1], ei));
+            if (l + 8 < L)
+                y[(size_t)(l + 8) * N + i0 + tp] =
+                    make_double2(mm64::to_double(hi[n][2], lo[n][2], er), mm64::to_double(hi[n][3], lo[n][3], ei));
         }
     }
 }
@@ -247,69 +308,77 @@ __global__ void __launch_bounds__(256) k_tdse_potential(const double2* __restric
 // s_l = (-1)^ceil(l/2) converts this library's sine/cosine sign convention to
 // the spherical-wave coefficients of Ytilde, so (-i)^l s_l = 1 (even l) or i
 // (odd l).  A is the vector potential sample of this step.
-__global__ void __launch_bounds__(256) k_tdse_velocity(double2* c, const double* __restrict__ P,
+// half: exp(-i k^2 tau/4) by storage row, as the kinetic phase table of tau / 2.
+__global__ void __launch_bounds__(128) k_tdse_velocity(double2* c, const uint2* __restrict__ Pw,
                                                        const double* __restrict__ eta,
-                                                       const double* __restrict__ knl, double dk, int L,
-                                                       int N, const double* __restrict__ A, int aidx,
-                                                       double tau, int m0) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    double* Ps = reinterpret_cast<double*>(sm);                    // [L][L]
-    double2* xs = reinterpret_cast<double2*>(Ps + kLMax * kLMax);  // [L][TI]
-    double2* xe = xs + kLMax * TI;                                 // [L][TI]
-    const int n0 = 1 + blockIdx.x * TI;
-    const int tid = threadIdx.x;
-    for (int k = tid; k < L * L; k += blockDim.x) Ps[k] = P[k];
-    for (int k = tid; k < L * TI; k += blockDim.x) {   // gather, half kinetic phase, (-i)^l s_l
-        const int ch = k / TI, t = k % TI, l = m0 + ch;   // channel ch holds angular momentum l
-        const int n = n0 + t;
-        double2 v = make_double2(0.0, 0.0);
-        if (n <= N) {
-            const int sidx = (l & 1) ? (n % N) : n - 1;
-            const double km = knl ? knl[(size_t)l * N + sidx] : k_index(l, sidx, N) * dk;
-            double sn, cs;
-            sincos(-0.25 * km * km * tau, &sn, &cs);
-            v = cmul2(c[(size_t)ch * N + sidx], make_double2(cs, sn));
-            if (l & 1) v = make_double2(-v.y, v.x);   // times i
+                                                       const double2* __restrict__ half_phase, int per_l, double dk, int L,
+                                                       int N, const double* __restrict__ A, int aidx, double tau, int m0) {
+    __shared__ AngularShared sh;
+    const int n0 = 1 + blockIdx.x * TI, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int t = tid % TI, kq = tid / TI, L16 = (L + 15) & ~15, half = (L + 1) / 2;
+    auto slot = [&](int ch, int n, double2& ph) {   // storage of momentum n of channel ch, and its half kinetic phase
+        const int l = m0 + ch, sidx = (l & 1) ? (n % N) : n - 1;
+        ph = per_l ? half_phase[(size_t)l * N + sidx] : half_phase[(size_t)(l & 1) * N + phase_entry(l, sidx, N)];
+        return (size_t)ch * N + sidx;
+    };
+    double2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {   // gather, half kinetic phase, (-i)^l s_l
+        const int ch = 4 * kq + q;
+        v[q] = make_double2(0.0, 0.0);
+        if (ch < L) {
+            double2 ph;
+            const size_t at = slot(ch, n0 + t, ph);
+            v[q] = cmul2(c[at], ph);
+            if ((m0 + ch) & 1) v[q] = make_double2(-v[q].y, v[q].x);   // times i
         }
-        xs[k] = v;
     }
+    if (tid < 4 * TI) sh.ef[tid / (2 * TI)][tid % (2 * TI)] = 0;
+    for (int k = tid; k < (L16 - L) * TI; k += blockDim.x) sh.grid[L + k / TI][k % TI] = make_double2(0.0, 0.0);
     __syncthreads();
+    angular_digits(sh, 0, kq, t, v);
     const double Av = A ? A[aidx] : 0.0;
-    for (int k = tid; k < L * TI; k += blockDim.x) {   // to the angular grid, A . P phase
-        const int j = k / TI, t = k % TI;
-        double2 s = make_double2(0.0, 0.0);
-        for (int l = 0; l < L; ++l) {
-            const double pj = Ps[l * L + j];
-            const double2 v = xs[l * TI + t];
-            s.x = fma(pj, v.x, s.x);
-            s.y = fma(pj, v.y, s.y);
+    if (8 * warp < half) {   // to the angular grid, A . P phase (node pairs as in k_tdse_potential)
+        long long hi[2][4], lo[2][4];
+        mm64::block_product<2>(Pw + (size_t)warp * 16 * kLMax, kLMax, L16 / 16, &sh.dig[0][0][0], AB, lane, hi, lo);
+        const int g = lane >> 2, tq = lane & 3, j = 8 * warp + g, jm = L - 1 - j;
+        if (j < half) {
+            const double ej = eta[j];
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const int tp = 4 * n + tq, er = sh.ef[0][2 * tp], ei = sh.ef[0][2 * tp + 1];
+                const double2 a = make_double2(mm64::to_double(hi[n][0], lo[n][0], er), mm64::to_double(hi[n][1], lo[n][1], ei));
+                const double2 b = make_double2(mm64::to_double(hi[n][2], lo[n][2], er), mm64::to_double(hi[n][3], lo[n][3], ei));
+                double sn, cs;
+                sincos(Av * ((n0 + tp) * dk) * ej * tau, &sn, &cs);
+                sh.grid[j][tp] = cmul2(a, make_double2(cs, sn));
+                if (jm != j) sh.grid[jm][tp] = cmul2(b, make_double2(cs, -sn));
+            }
         }
-        const int n = n0 + t;
-        if (n <= N) {
-            double sn, cs;
-            sincos(Av * (n * dk) * eta[j] * tau, &sn, &cs);
-            s = cmul2(s, make_double2(cs, sn));
-        }
-        xe[k] = s;
     }
     __syncthreads();
-    for (int k = tid; k < L * TI; k += blockDim.x) {   // back to l, i^l s_l, half kinetic phase, scatter
-        const int ch = k / TI, t = k % TI, l = m0 + ch;
-        const int n = n0 + t;
-        if (n > N) continue;
-        double2 s = make_double2(0.0, 0.0);
-        for (int j = 0; j < L; ++j) {
-            const double pl = Ps[ch * L + j];
-            const double2 v = xe[j * TI + t];
-            s.x = fma(pl, v.x, s.x);
-            s.y = fma(pl, v.y, s.y);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = 4 * kq + q < L16 ? sh.grid[4 * kq + q][t] : make_double2(0.0, 0.0);
+    angular_digits(sh, 1, kq, t, v);
+    if (16 * warp < L) {   // back to l, i^l s_l, half kinetic phase, scatter
+        long long hi[2][4], lo[2][4];
+        mm64::block_product<2>(Pw + (size_t)(kLMax + warp * 16) * kLMax, kLMax, L16 / 16, &sh.dig[0][0][0], AB, lane, hi,
+                               lo);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const int tp = 4 * n + (lane & 3), er = sh.ef[1][2 * tp], ei = sh.ef[1][2 * tp + 1];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int ch = 16 * warp + (lane >> 2) + 8 * q;
+                if (ch >= L) continue;
+                double2 s = make_double2(mm64::to_double(hi[n][2 * q], lo[n][2 * q], er),
+                                         mm64::to_double(hi[n][2 * q + 1], lo[n][2 * q + 1], ei));
+                if ((m0 + ch) & 1) s = make_double2(s.y, -s.x);   // times -i
+                double2 ph;
+                const size_t at = slot(ch, n0 + tp, ph);
+                c[at] = cmul2(s, ph);
+            }
         }
-        if (l & 1) s = make_double2(s.y, -s.x);   // times -i
-        const int sidx = (l & 1) ? (n % N) : n - 1;
-        const double km = knl ? knl[(size_t)l * N + sidx] : k_index(l, sidx, N) * dk;
-        double sn, cs;
-        sincos(-0.25 * km * km * tau, &sn, &cs);
-        c[(size_t)ch * N + sidx] = cmul2(s, make_double2(cs, sn));
     }
 }
 
@@ -345,13 +414,13 @@ namespace {
 
 inline size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-int potential(const dsbt_tdse* t, const double2* x, double2* y, const double* E, int eidx, double ht,
-              const double2* aux, double gscale, double* gacc, cudaStream_t st) {
-    const size_t smem = (size_t)kLMax * kLMax * sizeof(double) + 3 * (size_t)kLMax * TI * sizeof(double2);
-    if (int rc0 = ensure_smem((const void*)k_tdse_potential, smem)) return rc0;
+// One angular pass with the samples e1 and (merged half steps) e2 >= 0; see k_tdse_potential.
+int potential(const dsbt_tdse* t, const double2* x, double2* y, const double* E, int e1, int e2, double ht,
+              cudaStream_t st, double2* grid_out = nullptr, const double2* grid_in = nullptr, double gscale = 0.0,
+              double* g1 = nullptr, double* g2 = nullptr) {
     ProfScope ps(kKTdsePot, st);
-    k_tdse_potential<<<(t->N + TI - 1) / TI, 256, smem, st>>>(x, y, t->P, t->V, t->rr, t->eta, t->L, t->N, E,
-                                                              eidx, ht, aux, gscale, gacc);
+    k_tdse_potential<<<t->N / TI, 128, 0, st>>>(x, y, t->Pw, t->V, t->rr, t->eta, t->L, t->N, E, e1, e2, ht, grid_out,
+                                                grid_in, gscale, g1, g2);
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -364,35 +433,26 @@ int observable(const dsbt_tdse* t, const double2* x, double2* lam, double rc, do
     return DSBT_OK;
 }
 
-// One forward step psi_in -> psi_out (tmp: one state of scratch).
-int step(const dsbt_tdse* t, const double2* in, double2* out, double2* tmp, const double* E, int eidx,
-         double tau, const int* counts, void* kws, size_t kws_b, cudaStream_t st) {
-    int rc = potential(t, in, tmp, E, eidx, 0.5 * tau, nullptr, 0.0, nullptr, st);
-    if (!rc) rc = kinetic_grouped_with_scratch(t->plan, counts, DSBT_C128, tau, tmp, out, kws, kws_b, st);
-    if (!rc) rc = potential(t, out, out, E, eidx, 0.5 * tau, nullptr, 0.0, nullptr, st);
-    return rc;
+// The kinetic step of one state with the phase table already in the workspace.
+int kinetic(const dsbt_tdse* t, const int* counts, const double2* x, double2* y, void* kws, size_t kws_b,
+            cudaStream_t st) {
+    return grouped_device_call(kKineticReady, t->plan, counts, DSBT_C128, 0.0, x, y, kws, kws_b, st);
 }
 
-// One velocity-gauge step (Eq. (81)): potential half step (U = V + E r eta),
-// forward DSBT, momentum-space middle (k_tdse_velocity), inverse DSBT,
-// potential half step.  c: one state of scratch for the coefficients.
-int step_velocity(const dsbt_tdse* t, const double2* in, double2* out, double2* tmp, double2* c,
-                  const double* E, const double* A, int idx, double tau, const int* counts, void* kws,
-                  size_t kws_b, cudaStream_t st) {
-    int rc = potential(t, in, tmp, E, idx, 0.5 * tau, nullptr, 0.0, nullptr, st);
-    if (!rc) rc = grouped_device_call(0, t->plan, counts, DSBT_C128, 0.0, tmp, c, kws, kws_b, st);
+// The momentum-space part of a velocity-gauge step (Eq. (81)): forward DSBT,
+// k_tdse_velocity, inverse DSBT (c: one state of scratch for the coefficients; the
+// workspace's phase table holds tau / 2).
+int momentum_part(const dsbt_tdse* t, const int* counts, const double2* x, double2* y, double2* c, const double* A,
+                  int idx, double tau, void* kws, size_t kws_b, cudaStream_t st) {
+    int rc = grouped_device_call(0, t->plan, counts, DSBT_C128, 0.0, x, c, kws, kws_b, st);
     if (rc) return rc;
     {
-        const size_t smem = (size_t)kLMax * kLMax * sizeof(double) + 2 * (size_t)kLMax * TI * sizeof(double2);
-        if (int rc0 = ensure_smem((const void*)k_tdse_velocity, smem)) return rc0;
         ProfScope ps(kKTdseAng, st);
-        k_tdse_velocity<<<(t->N + TI - 1) / TI, 256, smem, st>>>(c, t->P, t->eta, t->plan->knl, t->plan->dk,
-                                                                 t->L, t->N, A, idx, tau, t->m0);
+        k_tdse_velocity<<<t->N / TI, 128, 0, st>>>(c, t->Pw, t->eta, kinetic_phase_table(t->plan, kws, t->L), t->plan->knl != nullptr,
+                                                   t->plan->dk, t->L, t->N, A, idx, tau, t->m0);
         DSBT_CUDA_TRY(cudaGetLastError());
     }
-    rc = grouped_device_call(1, t->plan, counts, DSBT_C128, 0.0, c, out, kws, kws_b, st);
-    if (!rc) rc = potential(t, out, out, E, idx, 0.5 * tau, nullptr, 0.0, nullptr, st);
-    return rc;
+    return grouped_device_call(1, t->plan, counts, DSBT_C128, 0.0, c, y, kws, kws_b, st);
 }
 
 struct TdseWs {
@@ -466,17 +526,31 @@ extern "C" int dsbt_tdse_create_m(const dsbt_plan* plan, int L, int m, double ta
         rh[i] = (i + 0.5) * t->dr;
         Vh[i] = -Z / sqrt(rh[i] * rh[i] + a2);
     }
+    // words of P^T with the nodes in mirror pairs (row 16 m + g: node 8 m + g, row
+    // 16 m + 8 + g: its mirror; the middle node of an odd L once), then of P
+    std::vector<uint2> Pw((size_t)2 * kLMax * kLMax, mm64::fixed_a_host(0.0));
+    for (int r = 0; r < kLMax; ++r) {
+        const int j = 8 * (r / 16) + r % 8, node = (r & 8) ? L - 1 - j : j;
+        const bool on = j < (L + 1) / 2 && !((r & 8) && node == j);
+        for (int k = 0; k < L; ++k) {
+            if (on) Pw[(size_t)r * kLMax + k] = mm64::fixed_a_host(Ph[(size_t)k * L + node]);
+            if (r < L) Pw[(size_t)(kLMax + r) * kLMax + k] = mm64::fixed_a_host(Ph[(size_t)r * L + k]);
+        }
+    }
     bool ok = cudaMalloc((void**)&t->P, Ph.size() * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&t->Pw, Pw.size() * sizeof(uint2)) == cudaSuccess &&
               cudaMalloc((void**)&t->V, t->N * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&t->rr, t->N * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&t->eta, L * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMemcpy(t->P, Ph.data(), Ph.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaMemcpy(t->Pw, Pw.data(), Pw.size() * sizeof(uint2), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(t->V, Vh.data(), t->N * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(t->rr, rh.data(), t->N * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(t->eta, t->eta_h.data(), L * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         cudaFree(t->P);
+        cudaFree(t->Pw);
         cudaFree(t->V);
         cudaFree(t->rr);
         cudaFree(t->eta);
@@ -500,6 +574,7 @@ extern "C" int dsbt_tdse_destroy(dsbt_tdse* t) {
     if (!t) return DSBT_OK;
     cudaDeviceSynchronize();
     cudaFree(t->P);
+    cudaFree(t->Pw);
     cudaFree(t->V);
     cudaFree(t->rr);
     cudaFree(t->eta);
@@ -542,14 +617,18 @@ extern "C" int dsbt_tdse_propagate(const dsbt_tdse* t, void* psi, const double* 
     for (int l = 0; l < t->L; ++l) counts[t->m0 + l] = 1;
     double2* x = (double2*)psi;
     const double tau = tau_sign * t->tau;
-    for (int s = 0; s < nsteps; ++s) {
-        // forward in time: sample s / hold; backward (tau < 0): the samples in reverse
-        const int eidx = (tau_sign > 0) ? s / hold : (nsteps - 1 - s) / hold;
-        rc = step(t, x, w.a, w.tmp, E, eidx, tau, counts.data(), w.kws, w.kws_b, st);
-        if (rc) return rc;
-        DSBT_CUDA_TRY(cudaMemcpyAsync(x, w.a, state_bytes(t), cudaMemcpyDeviceToDevice, st));
+    if (nsteps == 0) return DSBT_OK;
+    rc = kinetic_phase_fill(t->plan, w.kws, t->L, tau, st);
+    // forward in time: sample s / hold; backward (tau < 0): the samples in reverse
+    auto sample = [&](int s) { return (tau_sign > 0 ? s : nsteps - 1 - s) / hold; };
+    if (!rc) rc = potential(t, x, w.a, E, sample(0), -1, 0.5 * tau, st);
+    for (int s = 0; s < nsteps && !rc; ++s) {
+        rc = kinetic(t, counts.data(), w.a, w.tmp, w.kws, w.kws_b, st);
+        if (rc) break;
+        if (s + 1 < nsteps) rc = potential(t, w.tmp, w.a, E, sample(s), sample(s + 1), 0.5 * tau, st);
+        else rc = potential(t, w.tmp, x, E, sample(s), -1, 0.5 * tau, st);
     }
-    return DSBT_OK;
+    return rc;
 }
 
 extern "C" int dsbt_tdse_propagate_velocity(const dsbt_tdse* t, void* psi, const double* E, const double* A,
@@ -567,13 +646,17 @@ extern "C" int dsbt_tdse_propagate_velocity(const dsbt_tdse* t, void* psi, const
     for (int l = 0; l < t->L; ++l) counts[t->m0 + l] = 1;
     double2* x = (double2*)psi;
     const double tau = tau_sign * t->tau;
-    for (int s = 0; s < nsteps; ++s) {
-        const int idx = (tau_sign > 0) ? s / hold : (nsteps - 1 - s) / hold;
-        int rc = step_velocity(t, x, w.a, w.tmp, w.mu, E, A, idx, tau, counts.data(), w.kws, w.kws_b, st);
-        if (rc) return rc;
-        DSBT_CUDA_TRY(cudaMemcpyAsync(x, w.a, state_bytes(t), cudaMemcpyDeviceToDevice, st));
+    if (nsteps == 0) return DSBT_OK;
+    int rc = kinetic_phase_fill(t->plan, w.kws, t->L, 0.5 * tau, st);
+    auto sample = [&](int s) { return (tau_sign > 0 ? s : nsteps - 1 - s) / hold; };
+    if (!rc) rc = potential(t, x, w.a, E, sample(0), -1, 0.5 * tau, st);
+    for (int s = 0; s < nsteps && !rc; ++s) {
+        rc = momentum_part(t, counts.data(), w.a, w.tmp, w.mu, A, sample(s), tau, w.kws, w.kws_b, st);
+        if (rc) break;
+        if (s + 1 < nsteps) rc = potential(t, w.tmp, w.a, E, sample(s), sample(s + 1), 0.5 * tau, st);
+        else rc = potential(t, w.tmp, x, E, sample(s), -1, 0.5 * tau, st);
     }
-    return DSBT_OK;
+    return rc;
 }
 
 extern "C" int dsbt_tdse_observable(const dsbt_tdse* t, const void* psi, double r_cut, double* out,
@@ -600,50 +683,55 @@ extern "C" int dsbt_tdse_gradient(const dsbt_tdse* t, const void* psi0, const do
     const size_t sstride = a256(sb) / sizeof(double2);
     std::vector<int> counts(t->plan->l_max + 1, 0);
     for (int l = 0; l < t->L; ++l) counts[t->m0 + l] = 1;
-    const double tau = t->tau;
-    // forward sweep with checkpoints every K steps
-    DSBT_CUDA_TRY(cudaMemcpyAsync(w.ckpt, psi0, sb, cudaMemcpyDeviceToDevice, st));
-    DSBT_CUDA_TRY(cudaMemcpyAsync(w.lam, psi0, sb, cudaMemcpyDeviceToDevice, st));
-    for (int s = 0; s < nsteps; ++s) {
-        rc = step(t, w.lam, w.a, w.tmp, E, s / hold, tau, counts.data(), w.kws, w.kws_b, st);
-        if (rc) return rc;
-        std::swap(w.lam, w.a);
-        if ((s + 1) % K == 0)
-            DSBT_CUDA_TRY(cudaMemcpyAsync(w.ckpt + (size_t)((s + 1) / K) * sstride, w.lam, sb,
-                                          cudaMemcpyDeviceToDevice, st));
-    }
-    // observable and final adjoint state lambda_S = Pi psi_S
+    const double tau = t->tau, ht = 0.5 * tau;
     DSBT_CUDA_TRY(cudaMemsetAsync(O, 0, sizeof(double), st));
-    rc = observable(t, w.lam, w.mu, r_cut, O, st);
-    if (rc) return rc;
-    std::swap(w.lam, w.mu);
     DSBT_CUDA_TRY(cudaMemsetAsync(dOdE, 0, (size_t)nsamples * sizeof(double), st));
+    if (nsteps == 0) return observable(t, (const double2*)psi0, nullptr, r_cut, O, st);
+    auto smp = [&](int s) { return s / hold; };
+    auto kin = [&](const double2* x, double2* y) { return kinetic(t, counts.data(), x, y, w.kws, w.kws_b, st); };
+    // forward sweep: a_s = Q_s psi_s, b_s = Kin a_s = psi_{s+1} before its half step;
+    // checkpoint k holds b_{kK-1} (k = 0: psi_0)
+    rc = kinetic_phase_fill(t->plan, w.kws, t->L, tau, st);
+    if (rc) return rc;
+    DSBT_CUDA_TRY(cudaMemcpyAsync(w.ckpt, psi0, sb, cudaMemcpyDeviceToDevice, st));
+    rc = potential(t, (const double2*)psi0, w.a, E, smp(0), -1, ht, st);
+    const double2* b = w.tmp;   // b_s of the latest step
+    for (int s = 0; s < nsteps && !rc; ++s) {
+        double2* to = (s + 1 < nsteps && (s + 1) % K == 0) ? w.ckpt + (size_t)((s + 1) / K) * sstride : w.tmp;
+        rc = kin(w.a, to);
+        b = to;
+        if (!rc && s + 1 < nsteps) rc = potential(t, b, w.a, E, smp(s), smp(s + 1), ht, st);
+    }
+    // psi_S, the observable, lambda_S = Pi psi_S and mu = Q_{S-1}^H lambda_S
+    if (!rc) rc = potential(t, b, w.lam, E, smp(nsteps - 1), -1, ht, st);
+    if (!rc) rc = observable(t, w.lam, w.mu, r_cut, O, st);
+    if (!rc) rc = potential(t, w.mu, w.mu, E, smp(nsteps - 1), -1, -ht, st);
+    if (rc) return rc;
     // backward sweep, one checkpoint segment at a time
     const int nseg = (nsteps + K - 1) / K;
     for (int seg = nseg - 1; seg >= 0; --seg) {
         const int s0 = seg * K, s1 = (s0 + K < nsteps) ? s0 + K : nsteps;
-        DSBT_CUDA_TRY(cudaMemcpyAsync(w.seg, w.ckpt + (size_t)seg * sstride, sb, cudaMemcpyDeviceToDevice, st));
-        for (int s = s0; s < s1; ++s) {
-            rc = step(t, w.seg + (size_t)(s - s0) * sstride, w.seg + (size_t)(s - s0 + 1) * sstride, w.tmp, E,
-                      s / hold, tau, counts.data(), w.kws, w.kws_b, st);
-            if (rc) return rc;
+        auto grid = [&](int s) { return w.seg + (size_t)(s - s0) * sstride; };   // P^T a_s
+        const double2* ck = w.ckpt + (size_t)seg * sstride;
+        if (seg < nseg - 1) rc = kinetic_phase_fill(t->plan, w.kws, t->L, tau, st);   // (the adjoint's table is in place)
+        if (!rc)
+            rc = s0 == 0 ? potential(t, ck, w.a, E, smp(0), -1, ht, st, grid(0))
+                         : potential(t, ck, w.a, E, smp(s0 - 1), smp(s0), ht, st, grid(s0));
+        for (int s = s0; s + 1 < s1 && !rc; ++s) {
+            rc = kin(w.a, w.tmp);
+            if (!rc) rc = potential(t, w.tmp, w.a, E, smp(s), smp(s + 1), ht, st, grid(s + 1));
         }
-        for (int s = s1 - 1; s >= s0; --s) {
-            const double2* psi_s = w.seg + (size_t)(s - s0) * sstride;
-            const double2* psi_s1 = w.seg + (size_t)(s - s0 + 1) * sstride;
-            double* g = dOdE + s / hold;
-            // a_s = Q_s psi_s
-            rc = potential(t, psi_s, w.a, E, s / hold, 0.5 * tau, nullptr, 0.0, nullptr, st);
-            // mu = Q_s^H lambda_{s+1};  dO/dE += tau Im <lambda_{s+1}, R psi_{s+1}>
-            if (!rc) rc = potential(t, w.lam, w.mu, E, s / hold, -0.5 * tau, psi_s1, tau, g, st);
-            // nu = Kin^H mu
-            if (!rc)
-                rc = kinetic_grouped_with_scratch(t->plan, counts.data(), DSBT_C128, -tau, w.mu, w.nu, w.kws,
-                                                  w.kws_b, st);
-            // lambda_s = Q_s^H nu;  dO/dE += tau Im <nu, R a_s>
-            if (!rc) rc = potential(t, w.nu, w.lam, E, s / hold, -0.5 * tau, w.a, tau, g, st);
-            if (rc) return rc;
+        if (!rc) rc = kinetic_phase_fill(t->plan, w.kws, t->L, -tau, st);
+        for (int s = s1 - 1; s >= s0 && !rc; --s) {
+            rc = kin(w.mu, w.nu);   // nu_s
+            if (rc) break;
+            // g_s into dO/dE_s and dO/dE_{s-1}; mu = Q_{s-1}^H Q_s^H nu_s
+            double* g = dOdE + smp(s);
+            rc = s > 0 ? potential(t, w.nu, w.mu, E, smp(s), smp(s - 1), -ht, st, nullptr, grid(s), tau, g,
+                                   dOdE + smp(s - 1))
+                       : potential(t, w.nu, nullptr, E, 0, -1, -ht, st, nullptr, grid(0), tau, g, nullptr);
         }
+        if (rc) return rc;
     }
     return DSBT_OK;
 }
