@@ -232,14 +232,13 @@ size_t fast_scratch_bytes(const dsbt_plan* p, int lines) {
 }
 
 void fast_operands(const dsbt_plan* p, const double** Q, const double** QT, const double** Qw, const double** QTw,
-                   const size_t** qoff, const double** beta,
+                   const double** beta,
                    const double** betaT, const double** near, const double** nearT, int* nleaf, int* levels) {
     const FastData* f = p->fast;
     *Q = f->Q;
     *QT = f->QT;
     *Qw = f->Qw;
     *QTw = f->QTw;
-    *qoff = f->qoff;
     *beta = f->beta;
     *betaT = f->betaT;
     *near = f->near;

@@ -60,6 +60,16 @@ constexpr int KM = 64;          // stored basis width
 constexpr int MAX_SEG = 12;
 constexpr int NARROW_MAX = 4;   // real lines of a group up to which the narrow form is used
 
+// Row tiles of a moment CTA over K = len columns: a warp has a latency of its own
+// per 16 columns, so long intervals share K between the warps (8 to 16 units each)
+// instead of giving each warp its own rows (64 units at 1024 columns made the
+// longest CTAs half of the launch's time).  Wide tiles keep their rows together:
+// there the digits of the lines cost more than a warp's latency.
+__host__ __device__ inline int moment_mt(int most, int len, int narrow) {
+    const int mt = !narrow ? 4 : (len >= 512 ? 1 : (len == 256 ? 2 : 4));
+    return mt < most ? mt : most;
+}
+
 enum Kind { kDense = 0, kMoments = 1, kFastRows = 2 };
 
 struct MmArgs {
@@ -69,7 +79,6 @@ struct MmArgs {
     const double* QT;
     const double* Qw;       // odd l: the first leaf of each level's Q, row 0 times sqrt(w_0) ...
     const double* QTw;      // ... and QT, column 0 times sqrt(w_0) (weights outside the inner loops: see fast64.cu)
-    const size_t* qoff;
     const double* beta;
     const double* betaT;
     const double* near;
@@ -82,6 +91,7 @@ struct MmArgs {
     int dir, in_cplx, out_cplx, per_l;
     int mt;                 // 16-row tiles per CTA at most: 1, 2 or 4
     int kind;
+    int narrow;             // this launch's form
     int npos;
     int gidx[kMaxGroups];        // groups of this launch, largest l first
     // CTAs: first (kFastRows forward) the completion tiles of all groups, comp0 the
@@ -89,7 +99,7 @@ struct MmArgs {
     // prefix: a round is one row block (or interval, longest first) of every group,
     // so the longest K ranges start first
     int comp0[kMaxGroups + 1];
-    int unit0[kMaxGroups + 1];
+    int unit0[3][kMaxGroups + 1];   // at 1, 2 and 4 row tiles per CTA
 };
 
 // A strided set of lines: line j, index k at base + (j >> 1) pair + (j & 1) odd + k step.
@@ -100,6 +110,8 @@ struct LineSet {
         return base + (size_t)(j >> 1) * pair + (size_t)(j & 1) * odd + (size_t)k * step;
     }
 };
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // A range of the tile's K axis: columns [k0, next segment's k0).
 struct Seg {
@@ -116,6 +128,9 @@ struct Tile {
     LineSet out;
 };
 
+// First entry of level j in the bases: levels below hold 64, 128, ... points of 64 functions.
+__device__ __forceinline__ size_t level_offset(int j) { return (size_t)KM * FB * ((1 << j) - 1); }
+
 // Moments of level j, interval i: levels below hold nleaf, nleaf / 2, ... intervals (a power of two).
 __device__ __forceinline__ double* moments_at(const MmArgs& a, int j, int i, int line) {
     return a.M + ((size_t)(2 * (a.nleaf - (a.nleaf >> j)) + i) * a.R + line) * KM;
@@ -127,7 +142,7 @@ __device__ __forceinline__ LineSet line_set(const GroupTable& g, int gi, int lin
 }
 
 // Fills the tile (called by warp 0; lane j < levels looks at level j).
-__device__ void make_tile(const MmArgs& a, const GroupTable& g, int gi, int round, int local, int line, int lane,
+__device__ void make_tile(const MmArgs& a, const GroupTable& g, int gi, int level, int round, int local, int line, int lane,
                           Tile& t) {
     const int l = g.l[gi], N = a.N, ne = n_extra(l), ne16 = (ne + 15) & ~15, l16 = (l + 15) & ~15;
     const LineSet in = line_set(g, gi, line, a.in_cplx, a.in, N);
@@ -151,16 +166,10 @@ __device__ void make_tile(const MmArgs& a, const GroupTable& g, int gi, int roun
     };
     LineSet out = full;
     if (a.kind == kMoments) {
-        // round: interval index over the levels, longest first; local: row block
-        const int mtiles = l16 >> 4;
-        mt = min(a.mt, mtiles > 2 ? 4 : mtiles);
-        int b = round, j = a.levels - 1;
-        while (b >= (a.nleaf >> (j + 1))) {
-            b -= a.nleaf >> (j + 1);
-            --j;
-        }
-        const int i = 2 * b, len = FB << j;
-        const size_t qoff = a.qoff[j];
+        // level and round: the interval; local: row block
+        const int mtiles = l16 >> 4, j = level, i = 2 * round, len = FB << j;
+        mt = min(moment_mt(a.mt, len, a.narrow), mtiles > 2 ? 4 : mtiles);
+        const size_t qoff = level_offset(j);
         row0 = local * mt * 16;
         nrow = min(mt * 16, l16 - row0);
         if (a.dir > 0)
@@ -206,7 +215,7 @@ __device__ void make_tile(const MmArgs& a, const GroupTable& g, int gi, int roun
                 add(a.nearT + (((size_t)l * a.nleaf + J) * FB + (row0 - jb)) * FB, FB, FB, 1, shifted(in, jb));
                 add_levels(lane < a.levels && !(i & 1) && i + 1 < (a.nleaf >> j),
                            (l & 1) && J == 0 ? a.Qw + ((size_t)j * FB + row0) * KM
-                                             : a.Q + a.qoff[j] + (size_t)(row0 - i * (FB << j)) * KM,
+                                             : a.Q + level_offset(j) + (size_t)(row0 - i * (FB << j)) * KM,
                            LineSet{moments_at(a, j, i, g.line0[gi] + line), 2 * KM, KM, 1});
             }
         }
@@ -251,13 +260,22 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     __half* dig = reinterpret_cast<__half*>(smem_raw);   // [ND][NL][BS]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, tq = lane & 3;
 
-    int round = -1, b = blockIdx.x;
+    int level = 0, round = -1, b = blockIdx.x;
     const int* pre = a.comp0;
     if (b >= a.comp0[a.npos]) {
         b -= a.comp0[a.npos];
-        pre = a.unit0;
-        round = b / a.unit0[a.npos];
-        b -= round * a.unit0[a.npos];
+        int mt = a.mt;
+        if (a.kind == kMoments) {   // the level, longest intervals first
+            for (level = a.levels - 1;; --level) {
+                mt = moment_mt(a.mt, FB << level, a.narrow);
+                const int n = (a.nleaf >> (level + 1)) * a.unit0[mt >> 1][a.npos];
+                if (b < n || level == 0) break;
+                b -= n;
+            }
+        }
+        pre = a.unit0[mt >> 1];
+        round = b / pre[a.npos];
+        b -= round * pre[a.npos];
     }
     int lo = 0, hi = a.npos;
     while (hi - lo > 1) {
@@ -269,7 +287,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     const int nl = g.line0[gi + 1] - g.line0[gi], lt = (nl + NL - 1) / NL;
     const int rel = b - pre[lo];
     const int line = (rel % lt) * NL, nline = min(NL, nl - line);
-    if (warp == 0) make_tile(a, g, gi, round, rel / lt, line, lane, t);
+    if (warp == 0) make_tile(a, g, gi, level, round, rel / lt, line, lane, t);
     if (tid < NL) ef[tid] = 0;
     __syncthreads();
     const int mt = t.mt, nrow = t.nrow, K = t.K, nseg = t.nseg;
@@ -286,16 +304,26 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     // every round.
     auto drain = [&]() {
         if (NARROW) {
-            // acc[i]: digit i of A, digit tq of the lines; acc[8 + i]: digit 4 + tq
+            // acc[i]: digit i of A, digit tq of the lines; acc[8 + i]: digit 4 + tq.
+            // Without the products of i + j > 7 the sums in units of digit 0 of the
+            // lines are multiples of 256^tq, so shifting them to the common unit is exact.
+            const int sh = 8 * tq;
 #pragma unroll
-            for (int i = 0; i < 12; ++i) {
-                const int s = i < 8 ? i + tq : (i - 8) + 4 + tq;
+            for (int c = 0; c < 4; ++c) {
+                long long h = 0, w = 0, w1 = 0;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const long long v = __float2int_rn(acc[i][c]);
-                    if (s < 4) shi[c] += v << (8 * (3 - s));
-                    else if (s < 8) slo[c] += v << (8 * (7 - s));
+                for (int i = 0; i < 8; ++i) {
+                    const long long v = __float2int_rn(i > 4 && i + tq > 7 ? 0.f : acc[i][c]);
+                    if (i < 4) h += v * (1ll << (8 * (3 - i)));
+                    else w += v * (1ll << (8 * (7 - i)));
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const long long v = __float2int_rn(i > 0 && i + tq > 3 ? 0.f : acc[8 + i][c]);
+                    w1 += v * (1ll << (8 * (3 - i)));
+                }
+                shi[c] += h >> sh;
+                slo[c] += ((w + w1) >> sh) + ((h & ((1ll << sh) - 1)) << (32 - sh));
             }
         } else {
 #pragma unroll
@@ -335,6 +363,19 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
         __syncthreads();
     }
 
+    // The A entries of a narrow tile come from HBM (each is used by one or two
+    // lines): ask for the first columns of every segment now, and for the rest in
+    // load, eight units ahead.
+    constexpr int AHEAD = 8 * 16;
+    if (NARROW) {
+        const int r = tid % (16 * mt);
+        for (int q = 0; q < nseg; ++q) {
+            const Seg& sg = t.seg[q];
+            const int len = min(AHEAD, (q + 1 < nseg ? t.seg[q + 1].k0 : K) - sg.k0);
+            for (int k = 16 * (tid / (16 * mt)); k < len; k += 16 * (THREADS / (16 * mt)))
+                if (r < nrow) prefetch_l2(sg.A + (size_t)r * sg.lda + k);
+        }
+    }
     const double* ap = nullptr;
     int lda = 0, fixed = 0, aseg = 0, aend = 0;
     ulonglong2 raw[4];   // row g: columns 4t .. 4t + 3; row g + 8
@@ -354,6 +395,10 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
         raw[1] = __ldg(r0 + 1);
         raw[2] = __ldg(r1);
         raw[3] = __ldg(r1 + 1);
+        if (NARROW && k + AHEAD < aend) {
+            prefetch_l2(ap + k + AHEAD);
+            prefetch_l2(ap + k + AHEAD + (size_t)8 * lda);
+        }
     };
     if (active && ks * 16 < K) load(ks * 16);
     for (int r0 = 0; r0 < K; r0 += KR) {
@@ -362,7 +407,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
         auto put_digits = [&](int j, int e, const double* v) { put_digits4(dig + (size_t)j * BS + tk, NL * BS, v, e); };
         const double* p = nullptr;
         int step = 0, pair = 0, odd = 0;
-        if (on) {
+        if (!NARROW && on) {
             const Seg& sg = t.seg[seg_at(r0 + tk)];
             p = sg.B.at(0, r0 + tk - sg.k0);
             step = sg.B.step, pair = sg.B.pair, odd = sg.B.odd;
@@ -372,21 +417,43 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
 #pragma unroll
             for (int c = 0; c < 4; ++c) v[c] = on && j < nline ? q[c * step] : 0.0;
         };
-        if (NARROW) {
+        if (NARROW) {   // the round's kr / 4 tasks of each line, spread over all threads
             double v[TASKS][4];
+            const int per = kr / 4;
+            int tj[TASKS], tkk[TASKS];
 #pragma unroll
-            for (int i = 0; i < TASKS; ++i) fetch(tline + i * LSTEP, v[i]);
+            for (int i = 0; i < TASKS; ++i) {
+                const int idx = tid + i * THREADS;
+                tj[i] = idx >= per;
+                tkk[i] = idx < 2 * per ? 4 * (idx - (idx >= per ? per : 0)) : -1;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[i][c] = 0.0;
+                if (tkk[i] >= 0 && tj[i] < nline) {
+                    const Seg& sg = t.seg[seg_at(r0 + tkk[i])];
+                    const double* q = sg.B.at(tj[i], r0 + tkk[i] - sg.k0);
+                    const int step = sg.B.step;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[i][c] = q[c * step];
+                }
+            }
             if (K <= KR) {   // the scales from these values
+                int e[2] = {0, 0};
 #pragma unroll
                 for (int i = 0; i < TASKS; ++i) {
-                    const int e = __reduce_max_sync(0xffffffffu, exponent4(v[i]));
-                    if (lane == 0) atomicMax(&ef[tline + i * LSTEP], e);
+                    const int x = exponent4(v[i]);
+                    e[0] = max(e[0], tj[i] ? 0 : x);
+                    e[1] = max(e[1], tj[i] ? x : 0);
+                }
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    e[q] = __reduce_max_sync(0xffffffffu, e[q]);
+                    if (lane == 0) atomicMax(&ef[q], e[q]);
                 }
                 __syncthreads();
             }
 #pragma unroll
             for (int i = 0; i < TASKS; ++i)
-                if (on) put_digits(tline + i * LSTEP, ef[tline + i * LSTEP], v[i]);
+                if (tkk[i] >= 0) put_digits4(dig + (size_t)tj[i] * BS + tkk[i], NL * BS, v[i], ef[tj[i]]);
         } else {
 #pragma unroll
             for (int i = 0; i < TASKS; i += 2) {
@@ -459,41 +526,52 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     }
 
     // ---- add the K groups of warps, through the digit buffer
-    if (NARROW) {   // first the digits of the lines, held by the four lanes of a row
+    if (NARROW) {
+        // first the digits of the lines, held by the four lanes of a row: lane tq ends
+        // with result tq (row g + 8 (tq / 2), line tq & 1) in place 0
+        const bool up = tq & 2, odd = tq & 1;
 #pragma unroll
-        for (int c = 0; c < NO; ++c)
-#pragma unroll
-            for (int o = 1; o < 4; o <<= 1) {
-                shi[c] += __shfl_xor_sync(0xffffffffu, shi[c], o);
-                slo[c] += __shfl_xor_sync(0xffffffffu, slo[c], o);
-            }
+        for (int c = 0; c < 2; ++c) {
+            const long long h = __shfl_xor_sync(0xffffffffu, up ? shi[c] : shi[c + 2], 2);
+            const long long w = __shfl_xor_sync(0xffffffffu, up ? slo[c] : slo[c + 2], 2);
+            shi[c] = (up ? shi[c + 2] : shi[c]) + h;
+            slo[c] = (up ? slo[c + 2] : slo[c]) + w;
+        }
+        const long long h = __shfl_xor_sync(0xffffffffu, odd ? shi[0] : shi[1], 1);
+        const long long w = __shfl_xor_sync(0xffffffffu, odd ? slo[0] : slo[1], 1);
+        shi[0] = (odd ? shi[1] : shi[0]) + h;
+        slo[0] = (odd ? slo[1] : slo[0]) + w;
     }
+    constexpr int NR = NARROW ? 1 : NO;   // results left per thread
     if (ks_n > 1) {
         longlong2* red = reinterpret_cast<longlong2*>(smem_raw);   // [warp - mt][result][lane]
         if (active && ks > 0)
 #pragma unroll
-            for (int c = 0; c < NO; ++c) red[((warp - mt) * NO + c) * 32 + lane] = make_longlong2(shi[c], slo[c]);
+            for (int c = 0; c < NR; ++c) red[((warp - mt) * NR + c) * 32 + lane] = make_longlong2(shi[c], slo[c]);
         __syncthreads();
         if (active && ks == 0)
             for (int q = 1; q < ks_n; ++q)
 #pragma unroll
-                for (int c = 0; c < NO; ++c) {
-                    const longlong2 v = red[(((q - 1) * mt + m) * NO + c) * 32 + lane];
+                for (int c = 0; c < NR; ++c) {
+                    const longlong2 v = red[(((q - 1) * mt + m) * NR + c) * 32 + lane];
                     shi[c] += v.x;
                     slo[c] += v.y;
                 }
     }
     if (!active || ks > 0) return;
 
-    // ---- store: a thread holds lines (2t, 2t + 1) of rows g and g + 8
+    // ---- store: wide threads hold lines (2t, 2t + 1) of rows g and g + 8
     const LineSet out = t.out;
     const int l = g.l[gi];
     const double2* ph = a.kind == kMoments ? nullptr : a.phase;
+    auto phase_of = [&](int r) {
+        const int row = t.phase_row + r;
+        return a.per_l ? ph[(size_t)l * a.N + row] : ph[(size_t)(l & 1) * a.N + phase_entry(l, row, a.N)];
+    };
     auto put = [&](int j, int r, double re, double im) {
         if (j >= nline) return;
         if (ph) {   // lines (j, j + 1) are the parts of one channel
-            const int row = t.phase_row + r;
-            const double2 w = a.per_l ? ph[(size_t)l * a.N + row] : ph[(size_t)(l & 1) * a.N + phase_entry(l, row, a.N)];
+            const double2 w = phase_of(r);
             const double s = re * w.x - im * w.y;
             im = re * w.y + im * w.x;
             re = s;
@@ -503,12 +581,14 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
         if (j + 1 < nline) *const_cast<double*>(out.at(j + 1, r)) = im;
     };
     if (NARROW) {
-        if (tq < 2) {
-            // row g (lane 0 of the row) or g + 8 (lane 1)
-            const long long h0 = tq ? shi[2] : shi[0], l0 = tq ? slo[2] : slo[0];
-            const long long h1 = tq ? shi[3] : shi[1], l1 = tq ? slo[3] : slo[1];
-            put(0, m * 16 + gr + 8 * tq, to_double(h0, l0, ef[0]), to_double(h1, l1, ef[1]));
+        const int j = tq & 1, r = m * 16 + gr + 4 * (tq & 2);
+        double v = to_double(shi[0], slo[0], ef[j]);
+        if (ph) {   // the lane's neighbour holds the channel's other part
+            const double o = __shfl_xor_sync(0xffffffffu, v, 1);
+            const double2 w = phase_of(r);
+            v = j ? o * w.y + v * w.x : v * w.x - o * w.y;
         }
+        if (j < nline) *const_cast<double*>(out.at(j, r)) = v;
     } else {
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
@@ -524,27 +604,31 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
 
 template <int NL>
 int launch(MmArgs a, const GroupTable& g, cudaStream_t st) {
+    a.narrow = NL == 2;
     // groups of this form, largest l first; returns the CTAs at a.mt row tiles each
     auto fill = [&]() {
         a.npos = 0;
-        a.comp0[0] = a.unit0[0] = 0;
+        a.comp0[0] = a.unit0[0][0] = a.unit0[1][0] = a.unit0[2][0] = 0;
         for (int gi = g.ngroups - 1; gi >= 0; --gi) {
-            const int nl = g.line0[gi + 1] - g.line0[gi], l = g.l[gi], lt = (nl + NL - 1) / NL;
+            const int nl = g.line0[gi + 1] - g.line0[gi], l = g.l[gi], lt = (nl + NL - 1) / NL, n = a.npos;
             if ((nl <= NARROW_MAX) != (NL == 2)) continue;
-            int per = 1;   // row blocks of a round
-            if (a.kind == kMoments) {
-                const int mtiles = (l + 15) / 16;
-                if (mtiles == 0) continue;
-                const int mt = std::min(a.mt, mtiles > 2 ? 4 : mtiles);
-                per = (mtiles + mt - 1) / mt;
+            const int mtiles = (l + 15) / 16;
+            if (a.kind == kMoments && mtiles == 0) continue;
+            a.gidx[n] = gi;
+            a.comp0[n + 1] = a.comp0[n] + (a.kind == kFastRows && a.dir > 0 ? lt * ((n_extra(l) + 15) / 16) : 0);
+            for (int q = 0; q < 3; ++q) {   // row blocks of a round at 1, 2, 4 row tiles
+                const int mt = std::min(1 << q, mtiles > 2 ? 4 : std::max(1, mtiles));
+                a.unit0[q][n + 1] = a.unit0[q][n] + lt * (a.kind == kMoments ? (mtiles + mt - 1) / mt : 1);
             }
-            a.gidx[a.npos] = gi;
-            a.comp0[a.npos + 1] = a.comp0[a.npos] + (a.kind == kFastRows && a.dir > 0 ? lt * ((n_extra(l) + 15) / 16) : 0);
-            a.unit0[a.npos + 1] = a.unit0[a.npos] + lt * per;
             ++a.npos;
         }
-        const int rounds = a.kind == kMoments ? a.nleaf - 1 : a.N / (16 * a.mt);   // used intervals: nleaf/2 + nleaf/4 + ...
-        return a.comp0[a.npos] + a.unit0[a.npos] * rounds;
+        int n = a.comp0[a.npos];
+        if (a.kind == kMoments)
+            for (int j = 0; j < a.levels; ++j)
+                n += (a.nleaf >> (j + 1)) * a.unit0[moment_mt(a.mt, FB << j, a.narrow) >> 1][a.npos];
+        else
+            n += a.N / (16 * a.mt) * a.unit0[a.mt >> 1][a.npos];
+        return n;
     };
     // rows per CTA: 64, or 32 or 16 (the warps then share the K range) until
     // every SM has two CTAs
@@ -593,7 +677,7 @@ int contract_f64(const dsbt_plan* p, const GroupTable& g, int dir, const double*
     a.per_l = p->knl != nullptr;   // phase table rows per l (corrected momenta) or by parity
     ProfScope ps(kKContract64, st);
     if (p->fast && fast_scratch) {
-        fast_operands(p, &a.Q, &a.QT, &a.Qw, &a.QTw, &a.qoff, &a.beta, &a.betaT, &a.near, &a.nearT, &a.nleaf, &a.levels);
+        fast_operands(p, &a.Q, &a.QT, &a.Qw, &a.QTw, &a.beta, &a.betaT, &a.near, &a.nearT, &a.nleaf, &a.levels);
         a.M = fast_scratch;
         a.kind = kMoments;
         if (int rc = launch_both(a, g, st)) return rc;

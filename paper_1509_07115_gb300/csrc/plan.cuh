@@ -149,8 +149,7 @@ size_t fast_scratch_bytes(const dsbt_plan* p, int lines);
 // beta [l][j][r][64] and [l][j][64][r], leaf blocks and transposes, all as
 // biased fixed-point words (mm64.cuh).
 void fast_operands(const dsbt_plan* p, const double** Q, const double** QT, const double** Qw, const double** QTw,
-                   const size_t** qoff, const double** beta,
-                   const double** betaT, const double** near, const double** nearT, int* nleaf, int* levels);
+                   const double** beta, const double** betaT, const double** near, const double** nearT, int* nleaf, int* levels);
 // Orthonormal basis [len][64] of the polynomials of degree < min(64, len) on
 // the points x_t = (2t+1)/len - 1 (Arnoldi with two Gram-Schmidt passes).
 void poly_basis(int len, std::vector<double>& Q);
