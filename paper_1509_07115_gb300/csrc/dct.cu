@@ -6,13 +6,17 @@
 
 namespace dsbt {
 
-// Grids with their own compile-time instantiation (the power-of-two sizes of
-// the common workloads); the rest take N at run time.
+// FP64 power-of-two grids have kernels of their own (dct64.cu).  FP32 grids with
+// their own compile-time instantiation: the power-of-two sizes of the common
+// workloads; the rest take N at run time.
 template <typename R, int MODE>
 static FwdKernel<R> fwd_kernel(int N) {
-    if (N == 2048) return k_dct_fwd<R, MODE, 1, 2048>;
-    if (N == 4096) return k_dct_fwd<R, MODE, 1, 4096>;
-    if (N == 8192) return k_dct_fwd<R, MODE, 1, 8192>;
+    if constexpr (sizeof(R) == 4) {
+        if (N == 2048) return k_dct_fwd<R, MODE, 1, 2048>;
+        if (N == 4096) return k_dct_fwd<R, MODE, 1, 4096>;
+        if (N == 8192) return k_dct_fwd<R, MODE, 1, 8192>;
+        if (odd_part(N) == 1) return k_dct_fwd<R, MODE, 1, 0>;
+    }
     switch (odd_part(N)) {
 #define DSBT_CASE(q) \
     case q: return k_dct_fwd<R, MODE, q, 0>;
@@ -24,9 +28,12 @@ static FwdKernel<R> fwd_kernel(int N) {
 
 template <typename R>
 static InvKernel<R> inv_kernel(int N) {
-    if (N == 2048) return k_dct_inv<R, 1, 2048>;
-    if (N == 4096) return k_dct_inv<R, 1, 4096>;
-    if (N == 8192) return k_dct_inv<R, 1, 8192>;
+    if constexpr (sizeof(R) == 4) {
+        if (N == 2048) return k_dct_inv<R, 1, 2048>;
+        if (N == 4096) return k_dct_inv<R, 1, 4096>;
+        if (N == 8192) return k_dct_inv<R, 1, 8192>;
+        if (odd_part(N) == 1) return k_dct_inv<R, 1, 0>;
+    }
     switch (odd_part(N)) {
 #define DSBT_CASE(q) \
     case q: return k_dct_inv<R, q, 0>;
@@ -39,6 +46,10 @@ static InvKernel<R> inv_kernel(int N) {
 int dct_forward_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in,
                     double* out, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
+    if (dct64_supported(p->N)) {
+        ProfScope ps(kKDctFwd, st);
+        return dct64(true, p, g, cplx, in, out, st);
+    }
     unsigned nb, th; size_t sm;
     FwdKernel<double> k = fwd_kernel<double, kPlain>(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);
@@ -67,6 +78,10 @@ int dct_forward_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
 int dct_inverse_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in,
                     double* out, cudaStream_t st) {
     if (nchannels(g) == 0) return DSBT_OK;
+    if (dct64_supported(p->N)) {
+        ProfScope ps(kKDctInv, st);
+        return dct64(false, p, g, cplx, in, out, st);
+    }
     unsigned nb, th; size_t sm;
     InvKernel<double> k = inv_kernel<double>(p->N);
     DSBT_CHECK_ARG(k != nullptr, "dct: N=%d not of the form 256 q, q <= 32", p->N);

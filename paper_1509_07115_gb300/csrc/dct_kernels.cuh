@@ -700,7 +700,7 @@ inline int odd_part(int N) {
     return q;
 }
 
-#define DSBT_DCT_Q_CASES(X) X(1) X(3) X(5) X(7) X(9) X(11) X(13) X(15) X(17) X(19) X(21) X(23) X(25) X(27) X(29) X(31)
+#define DSBT_DCT_Q_CASES(X) X(3) X(5) X(7) X(9) X(11) X(13) X(15) X(17) X(19) X(21) X(23) X(25) X(27) X(29) X(31)
 
 template <typename R>
 using FwdKernel = void (*)(GroupTable, int, int, const R*, void*, void*, float*, const typename Cx<R>::T*,

@@ -123,6 +123,10 @@ int dct_forward_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
 //   [2^12, 2^13)), scale[line] = 2^-e
 int dct_forward_f16(const dsbt_plan* p, const GroupTable& g, bool cplx, const float* in, __half* out_hi,
                     __half* out_lo, float* scale, cudaStream_t st);
+// Power-of-two grids in FP64, either direction (dct64.cu).
+bool dct64_supported(int N);
+int dct64(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in, double* out,
+          cudaStream_t st);
 // Inverse F_l^T from planar lines to the caller's layout.
 int dct_inverse_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in,
                     double* out, cudaStream_t st);
