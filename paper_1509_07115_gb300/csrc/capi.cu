@@ -409,14 +409,6 @@ const double2* kinetic_phase_table(const dsbt_plan* p, void* ws, int total_chann
     return carve(p, ws, total_channels, DSBT_C128).ph64;
 }
 
-// Grouped kinetic step with a scratch buffer supplied by the caller of this
-// function (the TDSE propagator's inner call).
-int kinetic_grouped_with_scratch(const dsbt_plan* p, const int* counts, int dtype, double tau,
-                                 const void* in, void* out, void* scratch, size_t scratch_bytes,
-                                 cudaStream_t st) {
-    return grouped_call(2, p, counts, dtype, tau, in, out, scratch, scratch_bytes, st);
-}
-
 }  // namespace dsbt
 
 using namespace dsbt;

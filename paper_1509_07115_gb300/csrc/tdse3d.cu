@@ -19,32 +19,34 @@
 // sample of the step (three components).  A field along z couples no m, and the
 // step then equals the fixed-m propagator's for every m.
 //
-// Adjoint (the gradient of O = sum_{r_i > r_cut} |psi_S|^2 over the field
-// samples): with a_s = Q_s psi_s, lambda_S = Pi psi_S (Pi the mask r_i > r_cut),
-// nu = Kin^H Q_s^H lambda_{s+1} and lambda_s = Q_s^H nu, the derivative of
-// Q_s by the component F_c is Y^H diag(-i r n_c tau/2) D Y, which gives
-//     dO/dF_{s,c} += tau Im <Y lambda_{s+1}, r n_c Y psi_{s+1}> + tau Im <Y nu, r n_c Y a_s>
-// (the same form as the m = 0 adjoint with eta replaced by n_c), accumulated
-// inside the adjoint angular kernel.
+// Adjacent half steps share the grid and Y is unitary, so Q_{s+1} Q_s = Y^H diag
+// exp(-i [2 V + r (F_s + F_{s+1}).n] tau/2) Y is one pass; a propagation has single
+// passes at its ends only.
+//
+// Adjoint (the gradient of O = sum_{r_i > r_cut} |psi_S|^2 over the field samples):
+// with a_s = Q_s psi_s, lambda_S = Pi psi_S (Pi the mask r_i > r_cut), nu_s =
+// Kin^H Q_s^H lambda_{s+1} and lambda_s = Q_s^H nu_s, the derivative by the
+// component F_c is
+//     dO/dF_{s,c} = tau Im <Y lambda_{s+1}, r n_c Y psi_{s+1}> + tau Im <Y nu_s, r n_c Y a_s>.
+// The diagonal r n_c commutes with Q_s on the grid, so the second term is g_{s,c} =
+// Im <Y lambda_s, r n_c Y psi_s> and the first g_{s+1,c} (g_S = 0: lambda_S = Pi
+// psi_S): dO/dF_s = tau (g_s + g_{s+1}), with g_s = Im <Y nu_s, r n_c Y a_s> from the
+// grid values of a_s that the forward pass of a segment stores.
 #include <math.h>
 
 #include <algorithm>
 #include <new>
 #include <vector>
 
+#include "mm64.cuh"
 #include "plan.cuh"
-
-namespace dsbt {
-int kinetic_grouped_with_scratch(const dsbt_plan* p, const int* counts, int dtype, double tau,
-                                 const void* in, void* out, void* scratch, size_t scratch_bytes,
-                                 cudaStream_t st);
-}
 
 struct dsbt_tdse3d {
     const dsbt_plan* plan;
     int L, M, NM, N, nchan;
     double tau;
-    double* P;        // [NM][L][L]: P^m (row i = l - |m|, column j), m = mi - M
+    uint2* Pw;        // [M + 1][2][32][32] fixed-point words (mm64.cuh) of P^|m| (row i = l - |m|, column j):
+                      // P^T by node pairs, then P
     int* map;         // [NM][L]: channel of (l = |m| + i, m)
     int* lch;         // [nchan]: l of each channel
     double* V;        // [N]
@@ -57,153 +59,243 @@ struct dsbt_tdse3d {
 namespace dsbt {
 namespace {
 
-constexpr int TI3 = 4;   // radial points per block of the angular kernel
+constexpr int TI3 = 4;    // radial points per block of the angular kernels: 8 real columns
+constexpr int L3 = 32;     // the largest L
+constexpr int AB3 = L3 + 16;   // halfs per digit row (mm64.cuh)
+constexpr int DIG3 = mm64::ND * 2 * TI3 * AB3;   // halfs of one warp's digits
 
-// y = Q x on TI3 radial points per block (x and y may alias): to the
-// (theta, phi) grid, the phase exp(-i [V + r F.n] ht), back.  Shared memory:
-// the channel values, G[m][j] and the grid values, each [.][TI3].  With aux
-// != nullptr (adjoint steps), also adds gscale * Im( sum conj(Y x) r n_c Y aux )
-// over the grid into gacc[c], c = x, y, z (ga: the grid values of aux).
-__global__ void __launch_bounds__(256) k_tdse3d_potential(const double2* x, double2* y, const double* __restrict__ P,
-                                                          const int* __restrict__ map, const double* __restrict__ V,
-                                                          const double* __restrict__ rr,
-                                                          const double* __restrict__ eta, int L, int M, int N,
-                                                          int nchan, const double* __restrict__ F, int fidx,
-                                                          double ht, const double2* __restrict__ aux, double gscale,
-                                                          double* gacc) {
+struct Angular3 {
+    const uint2* Pw;
+    const int* map;     // [NM][L]: channel of (l = |m| + i, m)
+    const double* eta;
+    int L, M, N;
+};
+
+// Shared memory: G[NM][L][TI3] and g[L][NM][TI3] complex (the warps' digits in place of g),
+// cos and sin of 2 pi k / NM, and per node pair and point the phase of all but the field
+// across z.
+__host__ __device__ inline size_t grid3(int L, int NM) { return (size_t)NM * L * TI3 * sizeof(double2); }
+__host__ __device__ inline size_t second3(int L, int NM) {
+    const size_t d = 4 * (size_t)DIG3 * sizeof(__half), g = grid3(L, NM);
+    return d > g ? d : g;
+}
+inline size_t smem3d(int L, int NM) {
+    return grid3(L, NM) + second3(L, NM) + (size_t)NM * sizeof(double2) + (size_t)L3 * TI3 * sizeof(double2);
+}
+
+__device__ __forceinline__ double2 cmul3(double2 a, double2 b) {
+    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
+// One m block: digits of the warp's values (lane = 4 kq + t holds rows 4 kq .. 4 kq + 3 of
+// point t) and the product with the words A[32][32]; put(row, t, value) takes the results.
+template <class Put>
+__device__ __forceinline__ void m_block(const double2* v, const uint2* A, __half* dig, int L, int lane, Put&& put) {
+    const int t = lane & 3, kq = lane >> 2;
+    const double re[4] = {v[0].x, v[1].x, v[2].x, v[3].x}, im[4] = {v[0].y, v[1].y, v[2].y, v[3].y};
+    int er = mm64::exponent4(re), ei = mm64::exponent4(im);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        er = max(er, __shfl_xor_sync(0xffffffffu, er, o));
+        ei = max(ei, __shfl_xor_sync(0xffffffffu, ei, o));
+    }
+    __syncwarp();   // the digits of the block before are used up
+    mm64::put_digits4(dig + (2 * t) * AB3 + 4 * kq, 2 * TI3 * AB3, re, er);
+    mm64::put_digits4(dig + (2 * t + 1) * AB3 + 4 * kq, 2 * TI3 * AB3, im, ei);
+    __syncwarp();
+    const int units = (L + 15) / 16, tq = lane & 3, g = lane >> 2;
+    // lane tq's columns 2 tq, 2 tq + 1 are point tq: its scales are this lane's own
+    for (int b = 0; b < units; ++b) {
+        long long hi[1][4], lo[1][4];
+        mm64::block_product<1>(A + (size_t)b * 16 * L3, L3, units, dig, AB3, lane, hi, lo);
+        put(16 * b + g, tq, make_double2(mm64::to_double(hi[0][0], lo[0][0], er), mm64::to_double(hi[0][1], lo[0][1], ei)));
+        put(16 * b + g + 8, tq, make_double2(mm64::to_double(hi[0][2], lo[0][2], er), mm64::to_double(hi[0][3], lo[0][3], ei)));
+    }
+}
+
+// Node of row r of the P^T words (rows g and g + 8 of a 16-row block: node 8 b + g and its
+// mirror), or -1.
+__host__ __device__ inline int pair_node(int r, int L) {
+    const int j = 8 * (r / 16) + r % 8;
+    if (j >= (L + 1) / 2) return -1;
+    const int node = (r & 8) ? L - 1 - j : j;
+    return (r & 8) && node == j ? -1 : node;
+}
+
+// G -> G = Y^H D Y G on the block's points, with the phi sums written out in real
+// arithmetic: the DFT of NM = 2M + 1 angles works on the sums and differences of m and -m
+// (and of the angles q and -q), a quarter of the products of complex sums, and one sine
+// and cosine of each of a = r st Fx cos phi_q +- r st Fy sin phi_q serves a node and its
+// mirror.  zph[j][t]: exp(-i u) / NM with u the phase of everything that does not depend on
+// phi.  ab = (ax, ay): the phase of an angle is rad[t] st (ax cos phi + ay sin phi).
+// grid_out / grid_in: as in k_tdse3d_potential; returns the thread's part of the sums.
+__device__ __forceinline__ void phi_part(const Angular3& a, double2* G, double2* g, const double2* cs, const double2* zph,
+                                         const double* rad, double ax, double ay, int i0, double2* grid_out,
+                                         const double2* __restrict__ grid_in, double* gsum) {
+    const int L = a.L, M = a.M, NM = 2 * M + 1, tid = threadIdx.x, half = (L + 1) / 2;
+    // sums and differences of m and -m (in place: m takes the sum, -m the difference)
+    for (int k = tid; k < M * L * TI3; k += blockDim.x) {
+        const int m = 1 + k / (L * TI3), c = k % (L * TI3);
+        double2 &p = G[(M + m) * L * TI3 + c], &n = G[(M - m) * L * TI3 + c];
+        const double2 x = p, y = n;
+        p = make_double2(x.x + y.x, x.y + y.y);
+        n = make_double2(x.x - y.x, x.y - y.y);
+    }
+    __syncthreads();
+    // task: a node pair, a point and q in 0 .. M (angles q and -q)
+    for (int k = tid; k < half * TI3 * (M + 1); k += blockDim.x) {
+        const int t = k % TI3, j = (k / TI3) % half, q = k / (TI3 * half), jm = L - 1 - j;
+        double2 v[2][2];   // [node, mirror][q, -q]
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const double2* col = G + (s ? jm : j) * TI3 + t;
+            double2 A = col[M * L * TI3], B = make_double2(0.0, 0.0);
+            int e = 0;
+            for (int m = 1; m <= M; ++m) {   // A += (G_m + G_-m) cos, B += (G_m - G_-m) sin (times i)
+                e += q;
+                if (e >= NM) e -= NM;
+                const double2 w = cs[e], p = col[(M + m) * L * TI3], d = col[(M - m) * L * TI3];
+                A.x = fma(w.x, p.x, A.x);
+                A.y = fma(w.x, p.y, A.y);
+                B.x = fma(w.y, d.x, B.x);
+                B.y = fma(w.y, d.y, B.y);
+            }
+            v[s][0] = make_double2(A.x - B.y, A.y + B.x);
+            v[s][1] = make_double2(A.x + B.y, A.y - B.x);
+        }
+        const double ct = a.eta[j], st = sqrt(fmax(0.0, 1.0 - ct * ct)), cp = cs[q].x, sp = cs[q].y;
+        const size_t at = ((size_t)j * NM + q) * a.N + i0 + t, atm = ((size_t)jm * NM + q) * a.N + i0 + t,
+                     neg = (size_t)(q ? NM - 2 * q : 0) * a.N;   // from angle q to -q
+        if (grid_in) {
+            const double r = rad[t];
+            auto part = [&](double2 x, double2 y) { return r * (x.x * y.y - x.y * y.x); };
+            const double w0 = part(v[0][0], grid_in[at]), w1 = q ? part(v[0][1], grid_in[at + neg]) : 0.0;
+            const double u0 = jm != j ? part(v[1][0], grid_in[atm]) : 0.0,
+                         u1 = jm != j && q ? part(v[1][1], grid_in[atm + neg]) : 0.0;
+            gsum[0] += st * cp * ((w0 + w1) + (u0 + u1));
+            gsum[1] += st * sp * ((w0 - w1) + (u0 - u1));
+            gsum[2] += ct * ((w0 + w1) - (u0 + u1));
+        }
+        const double x = rad[t] * st * ax * cp, y = rad[t] * st * ay * sp;
+        double s0, c0, s1, c1;
+        sincos(x + y, &s0, &c0);
+        if (q) sincos(x - y, &s1, &c1);
+        else s1 = s0, c1 = c0;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            if (s && jm == j) break;
+            const double2 z = zph[(s ? jm : j) * TI3 + t];
+            const double2 h0 = cmul3(cmul3(v[s][0], z), make_double2(c0, s0));
+            const double2 h1 = cmul3(cmul3(v[s][1], z), make_double2(c1, s1));
+            double2* o = g + (size_t)((s ? jm : j) * NM) * TI3 + t;
+            if (grid_out) {
+                grid_out[s ? atm : at] = h0;
+                if (q) grid_out[(s ? atm : at) + neg] = h1;
+            }
+            if (q == 0) {
+                o[0] = h0;
+            } else {
+                o[q * TI3] = make_double2(h0.x + h1.x, h0.y + h1.y);
+                o[(NM - q) * TI3] = make_double2(h0.x - h1.x, h0.y - h1.y);
+            }
+        }
+    }
+    __syncthreads();
+    // back over phi: G_m = sum_q exp(-i m phi_q) h_q, m and -m together
+    for (int k = tid; k < L * TI3 * (M + 1); k += blockDim.x) {
+        const int t = k % TI3, j = (k / TI3) % L, m = k / (TI3 * L);
+        const double2* col = g + (size_t)j * NM * TI3 + t;
+        double2 A = col[0], B = make_double2(0.0, 0.0);
+        int e = 0;
+        for (int q = 1; q <= M; ++q) {
+            e += m;
+            if (e >= NM) e -= NM;
+            const double2 w = cs[e], p = col[q * TI3], d = col[(NM - q) * TI3];
+            A.x = fma(w.x, p.x, A.x);
+            A.y = fma(w.x, p.y, A.y);
+            B.x = fma(w.y, d.x, B.x);
+            B.y = fma(w.y, d.y, B.y);
+        }
+        G[((size_t)(M + m) * L + j) * TI3 + t] = make_double2(A.x + B.y, A.y - B.x);
+        if (m) G[((size_t)(M - m) * L + j) * TI3 + t] = make_double2(A.x - B.y, A.y + B.x);
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ void cos_table(double2* cs, int NM) {
+    for (int k = threadIdx.x; k < NM; k += blockDim.x) {
+        double sn, c;
+        sincospi(2.0 * (double)k / NM, &sn, &c);
+        cs[k] = make_double2(c, sn);
+    }
+}
+
+// y = Y^H diag(exp(-i [w V + r (F_f1 + F_f2).n] ht)) Y x on TI3 radial points per block
+// (w = 2, or w = 1 and no second sample for f2 < 0; x and y may alias; y may be null).
+// grid_out: also stores the grid values [L][NM][N] after the phase, divided by NM.
+// grid_in (values stored so): adds gscale * sum Im(conj(Y x) r n_c Y aux) into g1[c] and,
+// unless null, g2[c], c = x, y, z.  The P^m products run on the tensor cores through
+// exact digits, one m a warp.  What bounds it is the FP64 pipe: the phi sums and the sines.
+__global__ void __launch_bounds__(128) k_tdse3d_potential(const double2* x, double2* y, const __grid_constant__ Angular3 a,
+                                                          const double* __restrict__ V, const double* __restrict__ rr,
+                                                          const double* __restrict__ F, int f1, int f2, double ht,
+                                                          double2* grid_out, const double2* __restrict__ grid_in,
+                                                          double gscale, double* g1, double* g2) {
     extern __shared__ __align__(16) unsigned char sm[];
-    const int NM = 2 * M + 1;
-    double2* xs = reinterpret_cast<double2*>(sm);   // [nchan][TI3]
-    double2* G = xs + (size_t)nchan * TI3;          // [NM][L][TI3]
-    double2* g = G + (size_t)NM * L * TI3;          // [L][NM][TI3]
-    double2* ph = g + (size_t)NM * L * TI3;         // [NM][NM]: Phi[m][q]
-    double2* ga = ph + (size_t)NM * NM;             // [L][NM][TI3]: grid values of aux (adjoint only)
-    __shared__ double red[3][8];
-    const int i0 = blockIdx.x * TI3, tid = threadIdx.x;
-    const double inv = rsqrt((double)NM);
-    for (int k = tid; k < NM * NM; k += blockDim.x) {
-        const int mi = k / NM, q = k % NM;
-        double sn, cs;
-        sincospi(2.0 * (double)((mi - M) * q) / NM, &sn, &cs);
-        ph[k] = make_double2(cs * inv, sn * inv);
+    const int L = a.L, M = a.M, NM = 2 * M + 1, N = a.N, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double2* G = reinterpret_cast<double2*>(sm);
+    double2* g = reinterpret_cast<double2*>(sm + grid3(L, NM));
+    __half* dig = reinterpret_cast<__half*>(g) + (size_t)warp * DIG3;
+    double2* cs = reinterpret_cast<double2*>(sm + grid3(L, NM) + second3(L, NM));
+    double2* zph = cs + NM;
+    __shared__ double red[3][4], rad[TI3];
+    const int i0 = blockIdx.x * TI3, t = lane & 3, kq = lane >> 2;
+    double f[3] = {0.0, 0.0, 0.0};
+    if (F)
+        for (int c = 0; c < 3; ++c) f[c] = F[3 * f1 + c] + (f2 >= 0 ? F[3 * f2 + c] : 0.0);
+    cos_table(cs, NM);
+    for (int k = tid; k < L * TI3; k += blockDim.x) {
+        const int j = k / TI3, i = i0 + k % TI3;
+        double sn, c;
+        sincos(-((f2 >= 0 ? 2.0 : 1.0) * V[i] + rr[i] * f[2] * a.eta[j]) * ht, &sn, &c);
+        zph[k] = make_double2(c / NM, sn / NM);
     }
-    if (aux) {   // Y aux -> ga, through the same buffers
-        for (int k = tid; k < nchan * TI3; k += blockDim.x) {
-            const int c = k / TI3, t = k % TI3, i = i0 + t;
-            xs[k] = (i < N) ? aux[(size_t)c * N + i] : make_double2(0.0, 0.0);
+    if (tid < TI3) rad[tid] = rr[i0 + tid];
+    for (int mi = warp; mi < NM; mi += 4) {   // G_m(eta_j) = sum_l P^m x_lm
+        double2 v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            v[c] = 4 * kq + c < L ? x[(size_t)a.map[mi * L + 4 * kq + c] * N + i0 + t] : make_double2(0.0, 0.0);
+        m_block(v, a.Pw + (size_t)abs(mi - M) * 2 * L3 * L3, dig, L, lane, [&](int r, int tp, double2 w) {
+            const int j = pair_node(r, L);
+            if (j >= 0) G[((size_t)mi * L + j) * TI3 + tp] = w;
+        });
+    }
+    __syncthreads();
+    double gs[3] = {0.0, 0.0, 0.0};
+    phi_part(a, G, g, cs, zph, rad, -f[0] * ht, -f[1] * ht, i0, grid_out, grid_in, gs);
+    if (grid_in) {   // block sums of the three components
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            for (int o = 16; o > 0; o >>= 1) gs[c] += __shfl_xor_sync(0xffffffffu, gs[c], o);
+            if (lane == 0) red[c][warp] = gs[c];
         }
         __syncthreads();
-        for (int k = tid; k < NM * L * TI3; k += blockDim.x) {
-            const int mi = k / (L * TI3), j = (k / TI3) % L, t = k % TI3;
-            const double* Pm = P + (size_t)mi * L * L;
-            double2 s = make_double2(0.0, 0.0);
-            for (int ii = 0; ii < L; ++ii) {
-                const double p = Pm[ii * L + j];
-                const double2 v = xs[map[mi * L + ii] * TI3 + t];
-                s.x = fma(p, v.x, s.x);
-                s.y = fma(p, v.y, s.y);
-            }
-            G[k] = s;
-        }
-        __syncthreads();
-        for (int k = tid; k < L * NM * TI3; k += blockDim.x) {
-            const int j = k / (NM * TI3), q = (k / TI3) % NM, t = k % TI3;
-            double2 s = make_double2(0.0, 0.0);
-            for (int mi = 0; mi < NM; ++mi) {
-                const double2 a = ph[mi * NM + q], v = G[(mi * L + j) * TI3 + t];
-                s.x = fma(a.x, v.x, fma(-a.y, v.y, s.x));
-                s.y = fma(a.x, v.y, fma(a.y, v.x, s.y));
-            }
-            ga[k] = s;
-        }
-        __syncthreads();
-    }
-    for (int k = tid; k < nchan * TI3; k += blockDim.x) {
-        const int c = k / TI3, t = k % TI3, i = i0 + t;
-        xs[k] = (i < N) ? x[(size_t)c * N + i] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    for (int k = tid; k < NM * L * TI3; k += blockDim.x) {   // G_m(eta_j) = sum_l P^m x_lm
-        const int mi = k / (L * TI3), j = (k / TI3) % L, t = k % TI3;
-        const double* Pm = P + (size_t)mi * L * L;
-        double2 s = make_double2(0.0, 0.0);
-        for (int ii = 0; ii < L; ++ii) {
-            const double p = Pm[ii * L + j];
-            const double2 v = xs[map[mi * L + ii] * TI3 + t];
-            s.x = fma(p, v.x, s.x);
-            s.y = fma(p, v.y, s.y);
-        }
-        G[k] = s;
-    }
-    __syncthreads();
-    const double Fx = F ? F[3 * fidx] : 0.0, Fy = F ? F[3 * fidx + 1] : 0.0, Fz = F ? F[3 * fidx + 2] : 0.0;
-    double gx = 0.0, gy = 0.0, gz = 0.0;
-    for (int k = tid; k < L * NM * TI3; k += blockDim.x) {   // grid values times the phase
-        const int j = k / (NM * TI3), q = (k / TI3) % NM, t = k % TI3, i = i0 + t;
-        double2 s = make_double2(0.0, 0.0);
-        for (int mi = 0; mi < NM; ++mi) {
-            const double2 a = ph[mi * NM + q], v = G[(mi * L + j) * TI3 + t];
-            s.x = fma(a.x, v.x, fma(-a.y, v.y, s.x));
-            s.y = fma(a.x, v.y, fma(a.y, v.x, s.y));
-        }
-        if (i < N) {
-            const double ct = eta[j], st = sqrt(fmax(0.0, 1.0 - ct * ct));
-            double sp, cp;
-            sincospi(2.0 * (double)q / NM, &sp, &cp);
-            if (aux) {   // Im(conj(Y x) Y aux) r n_c
-                const double2 va = ga[k];
-                const double im = rr[i] * (s.x * va.y - s.y * va.x);
-                gx += im * st * cp;
-                gy += im * st * sp;
-                gz += im * ct;
-            }
-            const double u = V[i] + rr[i] * (Fx * st * cp + Fy * st * sp + Fz * ct);
-            double sn, cs;
-            sincos(-u * ht, &sn, &cs);
-            s = make_double2(s.x * cs - s.y * sn, s.x * sn + s.y * cs);
-        }
-        g[k] = s;
-    }
-    if (aux) {   // block sums of the three components, one atomic each
-        for (int o = 16; o > 0; o >>= 1) {
-            gx += __shfl_xor_sync(0xffffffffu, gx, o);
-            gy += __shfl_xor_sync(0xffffffffu, gy, o);
-            gz += __shfl_xor_sync(0xffffffffu, gz, o);
-        }
-        if ((tid & 31) == 0) {
-            red[0][tid >> 5] = gx;
-            red[1][tid >> 5] = gy;
-            red[2][tid >> 5] = gz;
+        if (tid < 3) {
+            const double s = gscale * (red[tid][0] + red[tid][1] + red[tid][2] + red[tid][3]);
+            atomicAdd(g1 + tid, s);
+            if (g2) atomicAdd(g2 + tid, s);
         }
     }
-    __syncthreads();
-    if (aux && tid < 3) {
-        double tsum = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tsum += red[tid][w];
-        atomicAdd(gacc + tid, gscale * tsum);
-    }
-    for (int k = tid; k < NM * L * TI3; k += blockDim.x) {   // back over phi: sum_q conj(Phi[m][q]) g
-        const int mi = k / (L * TI3), j = (k / TI3) % L, t = k % TI3;
-        double2 s = make_double2(0.0, 0.0);
-        for (int q = 0; q < NM; ++q) {
-            const double2 a = ph[mi * NM + q], v = g[(j * NM + q) * TI3 + t];
-            s.x = fma(a.x, v.x, fma(a.y, v.y, s.x));
-            s.y = fma(a.x, v.y, fma(-a.y, v.x, s.y));
-        }
-        G[k] = s;
-    }
-    __syncthreads();
-    for (int k = tid; k < NM * L * TI3; k += blockDim.x) {   // back over theta: psi_lm = sum_j P^m G_m
-        const int mi = k / (L * TI3), ii = (k / TI3) % L, t = k % TI3, i = i0 + t;
-        const double* Pm = P + (size_t)mi * L * L + (size_t)ii * L;
-        double2 s = make_double2(0.0, 0.0);
-        for (int j = 0; j < L; ++j) {
-            const double p = Pm[j];
-            const double2 v = G[(mi * L + j) * TI3 + t];
-            s.x = fma(p, v.x, s.x);
-            s.y = fma(p, v.y, s.y);
-        }
-        if (i < N) y[(size_t)map[mi * L + ii] * N + i] = s;
+    if (!y) return;
+    for (int mi = warp; mi < NM; mi += 4) {   // back over theta: psi_lm = sum_j P^m G_m
+        double2 v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            v[c] = 4 * kq + c < L ? G[((size_t)mi * L + 4 * kq + c) * TI3 + t] : make_double2(0.0, 0.0);
+        m_block(v, a.Pw + ((size_t)abs(mi - M) * 2 + 1) * L3 * L3, dig, L, lane, [&](int r, int tp, double2 w) {
+            if (r < L) y[(size_t)a.map[mi * L + r] * N + i0 + tp] = w;
+        });
     }
 }
 
@@ -211,127 +303,87 @@ __global__ void __launch_bounds__(256) k_tdse3d_potential(const double2* x, doub
 // in place on the DSBT coefficients c[ch][s] at TI3 momentum slots
 // n = 1..N per block (k~_n = n dk; storage s = n - 1 for even l, s = n for odd
 // l with n = N at s = 0): the half kinetic phase exp(-i k^2 tau/4) with the
-// plan's momentum of (l, s); phi = Ytilde^H c with the factors (-i)^l s_l = 1
-// (even l) or i (odd l) of the modified harmonics (s_l: this library's
-// sine/cosine signs); phi *= exp(i k~_n (A . n) tau) on the (theta, phi) grid;
-// c = Ytilde phi with i^l s_l = 1 or -i; the half kinetic phase again.
-__global__ void __launch_bounds__(256) k_tdse3d_velocity(double2* c, const double* __restrict__ P,
-                                                         const int* __restrict__ map, const int* __restrict__ lch,
-                                                         const double* __restrict__ eta,
-                                                         const double* __restrict__ knl, double dk, int L, int M,
-                                                         int N, int nchan, const double* __restrict__ A, int aidx,
-                                                         double tau) {
+// plan's momentum of (l, s) (half_phase: the kinetic phase table of tau / 2);
+// phi = Ytilde^H c with the factors (-i)^l s_l = 1 (even l) or i (odd l) of the
+// modified harmonics (s_l: this library's sine/cosine signs); phi *= exp(i k~_n
+// (A . n) tau) on the (theta, phi) grid; c = Ytilde phi with i^l s_l = 1 or -i; the
+// half kinetic phase again.
+__global__ void __launch_bounds__(128) k_tdse3d_velocity(double2* c, const __grid_constant__ Angular3 a,
+                                                         const int* __restrict__ lch,
+                                                         const double2* __restrict__ half_phase, int per_l, double dk,
+                                                         const double* __restrict__ A, int aidx, double tau) {
     extern __shared__ __align__(16) unsigned char sm[];
-    const int NM = 2 * M + 1;
-    double2* xs = reinterpret_cast<double2*>(sm);   // [nchan][TI3]
-    double2* G = xs + (size_t)nchan * TI3;          // [NM][L][TI3]
-    double2* g = G + (size_t)NM * L * TI3;          // [L][NM][TI3]
-    double2* ph = g + (size_t)NM * L * TI3;         // [NM][NM]
-    const int n0 = 1 + blockIdx.x * TI3, tid = threadIdx.x;
-    const double inv = rsqrt((double)NM);
-    for (int k = tid; k < NM * NM; k += blockDim.x) {
-        const int mi = k / NM, q = k % NM;
-        double sn, cs;
-        sincospi(2.0 * (double)((mi - M) * q) / NM, &sn, &cs);
-        ph[k] = make_double2(cs * inv, sn * inv);
+    const int L = a.L, M = a.M, NM = 2 * M + 1, N = a.N, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double2* G = reinterpret_cast<double2*>(sm);
+    double2* g = reinterpret_cast<double2*>(sm + grid3(L, NM));
+    __half* dig = reinterpret_cast<__half*>(g) + (size_t)warp * DIG3;
+    double2* cs = reinterpret_cast<double2*>(sm + grid3(L, NM) + second3(L, NM));
+    double2* zph = cs + NM;
+    __shared__ double rad[TI3];
+    const int n0 = 1 + blockIdx.x * TI3, t = lane & 3, kq = lane >> 2;
+    double f[3] = {0.0, 0.0, 0.0};
+    if (A)
+        for (int q = 0; q < 3; ++q) f[q] = A[3 * aidx + q];
+    cos_table(cs, NM);
+    for (int k = tid; k < L * TI3; k += blockDim.x) {
+        double sn, cc;
+        sincos(f[2] * a.eta[k / TI3] * ((n0 + k % TI3) * dk) * tau, &sn, &cc);
+        zph[k] = make_double2(cc / NM, sn / NM);
     }
-    for (int k = tid; k < nchan * TI3; k += blockDim.x) {   // gather, half kinetic phase, (-i)^l s_l
-        const int ch = k / TI3, t = k % TI3, n = n0 + t, l = lch[ch];
-        double2 v = make_double2(0.0, 0.0);
-        if (n <= N) {
-            const int sidx = (l & 1) ? (n % N) : n - 1;
-            const double km = knl ? knl[(size_t)l * N + sidx] : k_index(l, sidx, N) * dk;
-            double sn, cs;
-            sincos(-0.25 * km * km * tau, &sn, &cs);
-            const double2 a = c[(size_t)ch * N + sidx];
-            v = make_double2(a.x * cs - a.y * sn, a.x * sn + a.y * cs);
-            if (l & 1) v = make_double2(-v.y, v.x);   // times i
-        }
-        xs[k] = v;
-    }
-    __syncthreads();
-    for (int k = tid; k < NM * L * TI3; k += blockDim.x) {
-        const int mi = k / (L * TI3), j = (k / TI3) % L, t = k % TI3;
-        const double* Pm = P + (size_t)mi * L * L;
-        double2 s = make_double2(0.0, 0.0);
-        for (int ii = 0; ii < L; ++ii) {
-            const double p = Pm[ii * L + j];
-            const double2 v = xs[map[mi * L + ii] * TI3 + t];
-            s.x = fma(p, v.x, s.x);
-            s.y = fma(p, v.y, s.y);
-        }
-        G[k] = s;
-    }
-    __syncthreads();
-    const double Ax = A ? A[3 * aidx] : 0.0, Ay = A ? A[3 * aidx + 1] : 0.0, Az = A ? A[3 * aidx + 2] : 0.0;
-    for (int k = tid; k < L * NM * TI3; k += blockDim.x) {   // A . p phase on the momentum grid
-        const int j = k / (NM * TI3), q = (k / TI3) % NM, t = k % TI3, n = n0 + t;
-        double2 s = make_double2(0.0, 0.0);
-        for (int mi = 0; mi < NM; ++mi) {
-            const double2 a = ph[mi * NM + q], v = G[(mi * L + j) * TI3 + t];
-            s.x = fma(a.x, v.x, fma(-a.y, v.y, s.x));
-            s.y = fma(a.x, v.y, fma(a.y, v.x, s.y));
-        }
-        if (n <= N) {
-            const double ct = eta[j], st = sqrt(fmax(0.0, 1.0 - ct * ct));
-            double sp, cp;
-            sincospi(2.0 * (double)q / NM, &sp, &cp);
-            const double an = Ax * st * cp + Ay * st * sp + Az * ct;
-            double sn, cs;
-            sincos(an * (n * dk) * tau, &sn, &cs);
-            s = make_double2(s.x * cs - s.y * sn, s.x * sn + s.y * cs);
-        }
-        g[k] = s;
-    }
-    __syncthreads();
-    for (int k = tid; k < NM * L * TI3; k += blockDim.x) {
-        const int mi = k / (L * TI3), j = (k / TI3) % L, t = k % TI3;
-        double2 s = make_double2(0.0, 0.0);
-        for (int q = 0; q < NM; ++q) {
-            const double2 a = ph[mi * NM + q], v = g[(j * NM + q) * TI3 + t];
-            s.x = fma(a.x, v.x, fma(a.y, v.y, s.x));
-            s.y = fma(a.x, v.y, fma(-a.y, v.x, s.y));
-        }
-        G[k] = s;
-    }
-    __syncthreads();
-    for (int k = tid; k < NM * L * TI3; k += blockDim.x) {   // back to (l, m), i^l s_l, half phase, scatter
-        const int mi = k / (L * TI3), ii = (k / TI3) % L, t = k % TI3, n = n0 + t;
-        if (n > N) continue;
-        const double* Pm = P + (size_t)mi * L * L + (size_t)ii * L;
-        double2 s = make_double2(0.0, 0.0);
-        for (int j = 0; j < L; ++j) {
-            const double p = Pm[j];
-            const double2 v = G[(mi * L + j) * TI3 + t];
-            s.x = fma(p, v.x, s.x);
-            s.y = fma(p, v.y, s.y);
-        }
-        const int ch = map[mi * L + ii], l = lch[ch];
-        if (l & 1) s = make_double2(s.y, -s.x);   // times -i
+    if (tid < TI3) rad[tid] = (n0 + tid) * dk;
+    auto slot = [&](int ch, int l, int n, double2& ph) {   // storage of momentum n, and its half kinetic phase
         const int sidx = (l & 1) ? (n % N) : n - 1;
-        const double km = knl ? knl[(size_t)l * N + sidx] : k_index(l, sidx, N) * dk;
-        double sn, cs;
-        sincos(-0.25 * km * km * tau, &sn, &cs);
-        c[(size_t)ch * N + sidx] = make_double2(s.x * cs - s.y * sn, s.x * sn + s.y * cs);
+        ph = per_l ? half_phase[(size_t)l * N + sidx] : half_phase[(size_t)(l & 1) * N + phase_entry(l, sidx, N)];
+        return (size_t)ch * N + sidx;
+    };
+    for (int mi = warp; mi < NM; mi += 4) {   // gather, half kinetic phase, (-i)^l s_l
+        double2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[q] = make_double2(0.0, 0.0);
+            if (4 * kq + q < L) {
+                const int ch = a.map[mi * L + 4 * kq + q], l = lch[ch];
+                double2 ph;
+                const size_t at = slot(ch, l, n0 + t, ph);
+                v[q] = cmul3(c[at], ph);
+                if (l & 1) v[q] = make_double2(-v[q].y, v[q].x);   // times i
+            }
+        }
+        m_block(v, a.Pw + (size_t)abs(mi - M) * 2 * L3 * L3, dig, L, lane, [&](int r, int tp, double2 w) {
+            const int j = pair_node(r, L);
+            if (j >= 0) G[((size_t)mi * L + j) * TI3 + tp] = w;
+        });
+    }
+    __syncthreads();
+    phi_part(a, G, g, cs, zph, rad, f[0] * tau, f[1] * tau, 0, nullptr, nullptr, nullptr);
+    for (int mi = warp; mi < NM; mi += 4) {   // back to (l, m), i^l s_l, half phase, scatter
+        double2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            v[q] = 4 * kq + q < L ? G[((size_t)mi * L + 4 * kq + q) * TI3 + t] : make_double2(0.0, 0.0);
+        m_block(v, a.Pw + ((size_t)abs(mi - M) * 2 + 1) * L3 * L3, dig, L, lane, [&](int r, int tp, double2 w) {
+            if (r >= L) return;
+            const int ch = a.map[mi * L + r], l = lch[ch];
+            if (l & 1) w = make_double2(w.y, -w.x);   // times -i
+            double2 ph;
+            const size_t at = slot(ch, l, n0 + tp, ph);
+            c[at] = cmul3(w, ph);
+        });
     }
 }
 
-size_t smem3d(const dsbt_tdse3d* t) {
-    return ((size_t)t->nchan * TI3 + 2 * (size_t)t->NM * t->L * TI3 + (size_t)t->NM * t->NM) * sizeof(double2);
-}
+Angular3 angular3(const dsbt_tdse3d* t) { return Angular3{t->Pw, t->map, t->eta, t->L, t->M, t->N}; }
 
-// Shared memory of the adjoint angular kernel: plus the grid values of aux.
-size_t smem3d_adj(const dsbt_tdse3d* t) { return smem3d(t) + (size_t)t->NM * t->L * TI3 * sizeof(double2); }
-
-int potential3d(const dsbt_tdse3d* t, const double2* x, double2* y, const double* F, int fidx, double ht,
-                cudaStream_t st, const double2* aux = nullptr, double gscale = 0.0, double* gacc = nullptr) {
-    const size_t smem = aux ? smem3d_adj(t) : smem3d(t);
+// One angular pass with the samples f1 and (merged half steps) f2 >= 0; see k_tdse3d_potential.
+int potential3d(const dsbt_tdse3d* t, const double2* x, double2* y, const double* F, int f1, int f2, double ht,
+                cudaStream_t st, double2* grid_out = nullptr, const double2* grid_in = nullptr, double gscale = 0.0,
+                double* g1 = nullptr, double* g2 = nullptr) {
+    const size_t smem = smem3d(t->L, t->NM);
     if (smem > 48 * 1024)
         if (int rc0 = ensure_smem((const void*)k_tdse3d_potential, smem)) return rc0;
     ProfScope ps(kKTdsePot, st);
-    k_tdse3d_potential<<<(t->N + TI3 - 1) / TI3, 256, smem, st>>>(x, y, t->P, t->map, t->V, t->rr, t->eta, t->L,
-                                                                  t->M, t->N, t->nchan, F, fidx, ht, aux, gscale,
-                                                                  gacc);
+    k_tdse3d_potential<<<t->N / TI3, 128, smem, st>>>(x, y, angular3(t), t->V, t->rr, F, f1, f2, ht, grid_out, grid_in,
+                                                      gscale, g1, g2);
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -368,14 +420,14 @@ int observable3d(const dsbt_tdse3d* t, const double2* x, double2* mask, double r
     return DSBT_OK;
 }
 
-int velocity3d(const dsbt_tdse3d* t, double2* c, const double* A, int aidx, cudaStream_t st) {
-    const size_t smem = smem3d(t);
+// Half kinetic phases from the table of tau / 2 in the workspace.
+int velocity3d(const dsbt_tdse3d* t, double2* c, const double* A, int aidx, void* kws, cudaStream_t st) {
+    const size_t smem = smem3d(t->L, t->NM);
     if (smem > 48 * 1024)
         if (int rc0 = ensure_smem((const void*)k_tdse3d_velocity, smem)) return rc0;
     ProfScope ps(kKTdseAng, st);
-    k_tdse3d_velocity<<<(t->N + TI3 - 1) / TI3, 256, smem, st>>>(c, t->P, t->map, t->lch, t->eta, t->plan->knl,
-                                                                 t->plan->dk, t->L, t->M, t->N, t->nchan, A, aidx,
-                                                                 t->tau);
+    k_tdse3d_velocity<<<t->N / TI3, 128, smem, st>>>(c, angular3(t), t->lch, kinetic_phase_table(t->plan, kws, t->nchan),
+                                                     t->plan->knl != nullptr, t->plan->dk, A, aidx, t->tau);
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -417,22 +469,29 @@ extern "C" int dsbt_tdse3d_create(const dsbt_plan* plan, int L, int M, double ta
             ++t->counts[l];
         }
     t->nchan = (int)t->chan_l.size();
-    std::vector<double> x, w, Pm, Pall((size_t)t->NM * L * L), rr(t->N);
+    std::vector<double> x, w, Pm, rr(t->N);
     tdse_gauss_legendre(L, x, w);
-    for (int mi = 0; mi < t->NM; ++mi) {
-        const int am = std::abs(mi - M);
-        tdse_angular_rows(L, am, x, w, Pm);
-        std::copy(Pm.begin(), Pm.end(), Pall.begin() + (size_t)mi * L * L);
+    std::vector<uint2> Pw((size_t)(M + 1) * 2 * L3 * L3, mm64::fixed_a_host(0.0));
+    for (int m = 0; m <= M; ++m) {
+        tdse_angular_rows(L, m, x, w, Pm);
+        uint2* pt = Pw.data() + (size_t)m * 2 * L3 * L3;
+        for (int r = 0; r < L3; ++r) {
+            const int node = pair_node(r, L);
+            for (int k = 0; k < L; ++k) {
+                if (node >= 0) pt[r * L3 + k] = mm64::fixed_a_host(Pm[(size_t)k * L + node]);
+                if (r < L) pt[(L3 + r) * L3 + k] = mm64::fixed_a_host(Pm[(size_t)r * L + k]);
+            }
+        }
     }
     const double dr = plan->r_max / plan->N;
     for (int i = 0; i < t->N; ++i) rr[i] = (i + 0.5) * dr;
-    bool ok = cudaMalloc((void**)&t->P, Pall.size() * sizeof(double)) == cudaSuccess &&
+    bool ok = cudaMalloc((void**)&t->Pw, Pw.size() * sizeof(uint2)) == cudaSuccess &&
               cudaMalloc((void**)&t->map, map.size() * sizeof(int)) == cudaSuccess &&
               cudaMalloc((void**)&t->lch, t->nchan * sizeof(int)) == cudaSuccess &&
               cudaMalloc((void**)&t->V, t->N * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&t->rr, t->N * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void**)&t->eta, L * sizeof(double)) == cudaSuccess;
-    ok = ok && cudaMemcpy(t->P, Pall.data(), Pall.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+    ok = ok && cudaMemcpy(t->Pw, Pw.data(), Pw.size() * sizeof(uint2), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(t->map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(t->lch, t->chan_l.data(), t->nchan * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(t->V, 0, t->N * sizeof(double)) == cudaSuccess &&
@@ -440,16 +499,10 @@ extern "C" int dsbt_tdse3d_create(const dsbt_plan* plan, int L, int M, double ta
          cudaMemcpy(t->eta, x.data(), L * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
-        cudaFree(t->P); cudaFree(t->map); cudaFree(t->lch); cudaFree(t->V); cudaFree(t->rr); cudaFree(t->eta);
+        cudaFree(t->Pw); cudaFree(t->map); cudaFree(t->lch); cudaFree(t->V); cudaFree(t->rr); cudaFree(t->eta);
         delete t;
         set_error("dsbt_tdse3d_create: device allocation or copy failed");
         return DSBT_ERR_NOMEM;
-    }
-    if (smem3d(t) > 200 * 1024) {
-        cudaFree(t->P); cudaFree(t->map); cudaFree(t->lch); cudaFree(t->V); cudaFree(t->rr); cudaFree(t->eta);
-        delete t;
-        set_error("dsbt_tdse3d_create: L=%d, M=%d need too much shared memory", L, M);
-        return DSBT_ERR_INVALID;
     }
     *out = t;
     return DSBT_OK;
@@ -458,7 +511,7 @@ extern "C" int dsbt_tdse3d_create(const dsbt_plan* plan, int L, int M, double ta
 extern "C" int dsbt_tdse3d_destroy(dsbt_tdse3d* t) {
     if (!t) return DSBT_OK;
     cudaDeviceSynchronize();
-    cudaFree(t->P);
+    cudaFree(t->Pw);
     cudaFree(t->map);
     cudaFree(t->lch);
     cudaFree(t->V);
@@ -504,14 +557,16 @@ extern "C" int dsbt_tdse3d_propagate(const dsbt_tdse3d* t, void* psi, const doub
     void* kws = base + 2 * a256((size_t)t->nchan * t->N * sizeof(double2));
     const size_t kws_b = dsbt_workspace_size(t->plan, t->nchan, DSBT_C128);
     double2* x = (double2*)psi;
-    for (int s = 0; s < nsteps; ++s) {
-        const int fidx = s / hold;
-        int rc = potential3d(t, x, tmp, F, fidx, 0.5 * t->tau, st);
-        if (!rc) rc = kinetic_grouped_with_scratch(t->plan, t->counts.data(), DSBT_C128, t->tau, tmp, x, kws, kws_b, st);
-        if (!rc) rc = potential3d(t, x, x, F, fidx, 0.5 * t->tau, st);
-        if (rc) return rc;
+    if (nsteps == 0) return DSBT_OK;
+    int rc = kinetic_phase_fill(t->plan, kws, t->nchan, t->tau, st);
+    if (!rc) rc = potential3d(t, x, tmp, F, 0, -1, 0.5 * t->tau, st);
+    for (int s = 0; s < nsteps && !rc; ++s) {
+        rc = grouped_device_call(kKineticReady, t->plan, t->counts.data(), DSBT_C128, 0.0, tmp, x, kws, kws_b, st);
+        if (rc) break;
+        if (s + 1 < nsteps) rc = potential3d(t, x, tmp, F, s / hold, (s + 1) / hold, 0.5 * t->tau, st);
+        else rc = potential3d(t, x, x, F, s / hold, -1, 0.5 * t->tau, st);
     }
-    return DSBT_OK;
+    return rc;
 }
 
 extern "C" int dsbt_tdse3d_propagate_velocity(const dsbt_tdse3d* t, void* psi, const double* F, const double* A,
@@ -530,16 +585,18 @@ extern "C" int dsbt_tdse3d_propagate_velocity(const dsbt_tdse3d* t, void* psi, c
     void* kws = base + 2 * sb;
     const size_t kws_b = dsbt_workspace_size(t->plan, t->nchan, DSBT_C128);
     double2* x = (double2*)psi;
-    for (int s = 0; s < nsteps; ++s) {
-        const int idx = s / hold;
-        int rc = potential3d(t, x, tmp, F, idx, 0.5 * t->tau, st);
-        if (!rc) rc = grouped_device_call(0, t->plan, t->counts.data(), DSBT_C128, 0.0, tmp, c, kws, kws_b, st);
-        if (!rc) rc = velocity3d(t, c, A, idx, st);
+    if (nsteps == 0) return DSBT_OK;
+    int rc = kinetic_phase_fill(t->plan, kws, t->nchan, 0.5 * t->tau, st);
+    if (!rc) rc = potential3d(t, x, tmp, F, 0, -1, 0.5 * t->tau, st);
+    for (int s = 0; s < nsteps && !rc; ++s) {
+        rc = grouped_device_call(0, t->plan, t->counts.data(), DSBT_C128, 0.0, tmp, c, kws, kws_b, st);
+        if (!rc) rc = velocity3d(t, c, A, s / hold, kws, st);
         if (!rc) rc = grouped_device_call(1, t->plan, t->counts.data(), DSBT_C128, 0.0, c, x, kws, kws_b, st);
-        if (!rc) rc = potential3d(t, x, x, F, idx, 0.5 * t->tau, st);
-        if (rc) return rc;
+        if (rc) break;
+        if (s + 1 < nsteps) rc = potential3d(t, x, tmp, F, s / hold, (s + 1) / hold, 0.5 * t->tau, st);
+        else rc = potential3d(t, x, x, F, s / hold, -1, 0.5 * t->tau, st);
     }
-    return DSBT_OK;
+    return rc;
 }
 
 namespace dsbt {
@@ -588,8 +645,6 @@ extern "C" int dsbt_tdse3d_gradient(const dsbt_tdse3d* t, const void* psi0, cons
     const size_t need = dsbt_tdse3d_gradient_workspace_size(t, nsteps, K);
     DSBT_CHECK_ARG(workspace != nullptr && workspace_bytes >= need,
                    "dsbt_tdse3d_gradient: workspace too small (need %zu bytes)", need);
-    DSBT_CHECK_ARG(smem3d_adj(t) <= 220 * 1024, "dsbt_tdse3d_gradient: L=%d, M=%d need too much shared memory",
-                   t->L, t->M);
     cudaStream_t st = (cudaStream_t)stream;
     double2 *ck, *seg, *a, *mu, *nu, *lam;
     void* kws;
@@ -599,52 +654,56 @@ extern "C" int dsbt_tdse3d_gradient(const dsbt_tdse3d* t, const void* psi0, cons
     const size_t stride = a256(sb) / sizeof(double2);
     const double tau = t->tau, ht = 0.5 * tau;
     const int* counts = t->counts.data();
-    // one step x -> y (Q Kin Q); tmp is clobbered
-    auto step = [&](const double2* x, double2* y, double2* tmp, int fidx) {
-        int rc = potential3d(t, x, tmp, F, fidx, ht, st);
-        if (!rc) rc = kinetic_grouped_with_scratch(t->plan, counts, DSBT_C128, tau, tmp, y, kws, kws_b, st);
-        if (!rc) rc = potential3d(t, y, y, F, fidx, ht, st);
-        return rc;
-    };
-    // forward sweep with checkpoints every K steps
-    DSBT_CUDA_TRY(cudaMemcpyAsync(ck, psi0, sb, cudaMemcpyDeviceToDevice, st));
-    DSBT_CUDA_TRY(cudaMemcpyAsync(lam, psi0, sb, cudaMemcpyDeviceToDevice, st));
-    for (int s = 0; s < nsteps; ++s) {
-        int rc = step(lam, a, mu, s / hold);
-        if (rc) return rc;
-        std::swap(lam, a);
-        if ((s + 1) % K == 0)
-            DSBT_CUDA_TRY(cudaMemcpyAsync(ck + (size_t)((s + 1) / K) * stride, lam, sb, cudaMemcpyDeviceToDevice, st));
-    }
-    // observable and lambda_S = Pi psi_S
     DSBT_CUDA_TRY(cudaMemsetAsync(O, 0, sizeof(double), st));
-    int rc = observable3d(t, lam, mu, r_cut, O, st);
-    if (rc) return rc;
-    std::swap(lam, mu);
     DSBT_CUDA_TRY(cudaMemsetAsync(dOdF, 0, (size_t)3 * nsamples * sizeof(double), st));
+    if (nsteps == 0) return observable3d(t, (const double2*)psi0, nullptr, r_cut, O, st);
+    auto smp = [&](int s) { return s / hold; };
+    auto kin = [&](const double2* x, double2* y) {
+        return grouped_device_call(kKineticReady, t->plan, counts, DSBT_C128, 0.0, x, y, kws, kws_b, st);
+    };
+    // forward sweep: a_s = Q_s psi_s, b_s = Kin a_s = psi_{s+1} before its half step;
+    // checkpoint k holds b_{kK-1} (k = 0: psi_0)
+    int rc = kinetic_phase_fill(t->plan, kws, t->nchan, tau, st);
+    if (rc) return rc;
+    DSBT_CUDA_TRY(cudaMemcpyAsync(ck, psi0, sb, cudaMemcpyDeviceToDevice, st));
+    rc = potential3d(t, (const double2*)psi0, a, F, smp(0), -1, ht, st);
+    const double2* b = nu;   // b_s of the latest step
+    for (int s = 0; s < nsteps && !rc; ++s) {
+        double2* to = (s + 1 < nsteps && (s + 1) % K == 0) ? ck + (size_t)((s + 1) / K) * stride : nu;
+        rc = kin(a, to);
+        b = to;
+        if (!rc && s + 1 < nsteps) rc = potential3d(t, b, a, F, smp(s), smp(s + 1), ht, st);
+    }
+    // psi_S, the observable, lambda_S = Pi psi_S and mu = Q_{S-1}^H lambda_S
+    if (!rc) rc = potential3d(t, b, lam, F, smp(nsteps - 1), -1, ht, st);
+    if (!rc) rc = observable3d(t, lam, mu, r_cut, O, st);
+    if (!rc) rc = potential3d(t, mu, mu, F, smp(nsteps - 1), -1, -ht, st);
+    if (rc) return rc;
     // backward sweep, one checkpoint segment at a time
     const int nseg = (nsteps + K - 1) / K;
     for (int sg = nseg - 1; sg >= 0; --sg) {
         const int s0 = sg * K, s1 = (s0 + K < nsteps) ? s0 + K : nsteps;
-        DSBT_CUDA_TRY(cudaMemcpyAsync(seg, ck + (size_t)sg * stride, sb, cudaMemcpyDeviceToDevice, st));
-        for (int s = s0; s < s1; ++s) {
-            rc = step(seg + (size_t)(s - s0) * stride, seg + (size_t)(s - s0 + 1) * stride, a, s / hold);
-            if (rc) return rc;
+        auto grid = [&](int s) { return seg + (size_t)(s - s0) * stride; };   // grid values of a_s
+        const double2* c = ck + (size_t)sg * stride;
+        if (sg < nseg - 1) rc = kinetic_phase_fill(t->plan, kws, t->nchan, tau, st);   // (the adjoint's table is in place)
+        if (!rc)
+            rc = s0 == 0 ? potential3d(t, c, a, F, smp(0), -1, ht, st, grid(0))
+                         : potential3d(t, c, a, F, smp(s0 - 1), smp(s0), ht, st, grid(s0));
+        for (int s = s0; s + 1 < s1 && !rc; ++s) {
+            rc = kin(a, nu);
+            if (!rc) rc = potential3d(t, nu, a, F, smp(s), smp(s + 1), ht, st, grid(s + 1));
         }
-        for (int s = s1 - 1; s >= s0; --s) {
-            const double2* psi_s = seg + (size_t)(s - s0) * stride;
-            const double2* psi_s1 = seg + (size_t)(s - s0 + 1) * stride;
-            double* g = dOdF + 3 * (size_t)(s / hold);
-            // a_s = Q_s psi_s
-            rc = potential3d(t, psi_s, a, F, s / hold, ht, st);
-            // mu = Q_s^H lambda_{s+1};  dO/dF += tau Im <Y lambda_{s+1}, r n Y psi_{s+1}>
-            if (!rc) rc = potential3d(t, lam, mu, F, s / hold, -ht, st, psi_s1, tau, g);
-            // nu = Kin^H mu
-            if (!rc) rc = kinetic_grouped_with_scratch(t->plan, counts, DSBT_C128, -tau, mu, nu, kws, kws_b, st);
-            // lambda_s = Q_s^H nu;  dO/dF += tau Im <Y nu, r n Y a_s>
-            if (!rc) rc = potential3d(t, nu, lam, F, s / hold, -ht, st, a, tau, g);
-            if (rc) return rc;
+        if (!rc) rc = kinetic_phase_fill(t->plan, kws, t->nchan, -tau, st);
+        for (int s = s1 - 1; s >= s0 && !rc; --s) {
+            rc = kin(mu, nu);   // nu_s
+            if (rc) break;
+            // g_s into dO/dF_s and dO/dF_{s-1}; mu = Q_{s-1}^H Q_s^H nu_s
+            double* g = dOdF + 3 * (size_t)smp(s);
+            rc = s > 0 ? potential3d(t, nu, mu, F, smp(s), smp(s - 1), -ht, st, nullptr, grid(s), tau, g,
+                                     dOdF + 3 * (size_t)smp(s - 1))
+                       : potential3d(t, nu, nullptr, F, 0, -1, -ht, st, nullptr, grid(0), tau, g, nullptr);
         }
+        if (rc) return rc;
     }
     return DSBT_OK;
 }
