@@ -401,6 +401,20 @@ int grouped_device_call(int which, const dsbt_plan* p, const int* counts, int dt
     return grouped_call(which, p, counts, dtype, tau, in, out, ws, ws_b, st, uoff);
 }
 
+int real_step(const dsbt_plan* p, int l, int nchan, const double* in, double* b, double* out, const double* row_scale,
+              void* ws, size_t ws_b, cudaStream_t st) {
+    int rc = check_common(p, DSBT_F64, in, b, ws, ws_b, nchan);
+    GroupTable g;
+    if (!rc) rc = build_groups(p, &nchan, 1, &l, DSBT_F64, g);
+    if (rc) return rc;
+    Workspace w = carve(p, ws, nchan, DSBT_F64);
+    rc = dct_forward_f64(p, g, false, in, w.f64a, st);
+    if (!rc) rc = contract_f64(p, g, +1, w.f64a, 0, b, 0, nullptr, st, w.fast, row_scale);
+    if (!rc) rc = contract_f64(p, g, -1, b, 0, w.f64a, 0, nullptr, st, w.fast);
+    if (!rc) rc = dct_inverse_f64(p, g, false, w.f64a, out, st);
+    return rc;
+}
+
 int kinetic_phase_fill(const dsbt_plan* p, void* ws, int total_channels, double tau, cudaStream_t st) {
     return fill_phase64(p, carve(p, ws, total_channels, DSBT_C128), tau, st);
 }

@@ -34,8 +34,10 @@
 //   narrow  2 lines a tile, the 8 digits of both lines as 16 columns, so one
 //           digit of A meets all digits of the lines in two instructions (12
 //           instead of 36): bound by turning A into digits and by reading it
-// Groups of up to 4 lines take the narrow form (two tiles of 12 instructions
-// against 36).
+// A 16 x 16 block of A costs a warp about 300 issue slots and 12 matrix
+// instructions per two lines (narrow), 250 and 72 per sixteen (wide): groups of up to 4
+// lines take the narrow form, and groups of up to 16 while the call leaves SMs idle
+// (5 lines of 1280 points: 49 us wide).
 //
 // Measured on a GB300, forward + inverse contraction of one call (before: FP64
 // multiply-adds on the same schemes):
@@ -58,7 +60,6 @@ constexpr int THREADS = 128;
 constexpr int FB = 64;          // leaf of the interval scheme
 constexpr int KM = 64;          // stored basis width
 constexpr int MAX_SEG = 12;
-constexpr int NARROW_MAX = 4;   // real lines of a group up to which the narrow form is used
 
 // Row tiles of a moment CTA over K = len columns: a warp has a latency of its own
 // per 16 columns, so long intervals share K between the warps (8 to 16 units each)
@@ -87,11 +88,13 @@ struct MmArgs {
     const double* in;
     double* out;
     const double2* phase;
+    const double* row_scale;   // real factor per output row, or null
     int N, nleaf, levels, R;
     int dir, in_cplx, out_cplx, per_l;
     int mt;                 // 16-row tiles per CTA at most: 1, 2 or 4
     int kind;
-    int narrow;             // this launch's form
+    int narrow;             // this launch's form ...
+    int narrow_max;         // ... and the most lines of a group that the narrow one takes
     int npos;
     int gidx[kMaxGroups];        // groups of this launch, largest l first
     // CTAs: first (kFastRows forward) the completion tiles of all groups, comp0 the
@@ -378,7 +381,9 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     }
     const double* ap = nullptr;
     int lda = 0, fixed = 0, aseg = 0, aend = 0;
-    ulonglong2 raw[4];   // row g: columns 4t .. 4t + 3; row g + 8
+    // Row g: columns 4t .. 4t + 3; row g + 8.  (Two units ahead, at three CTAs an SM
+    // instead of four, was 10 % slower for the narrow form.)
+    ulonglong2 raw[4];
     // loads this thread's A entries of the unit at column k (units of a warp come in increasing k)
     auto load = [&](int k) {
         if (k >= aend) {
@@ -564,6 +569,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     const LineSet out = t.out;
     const int l = g.l[gi];
     const double2* ph = a.kind == kMoments ? nullptr : a.phase;
+    const double* rs = a.kind == kMoments ? nullptr : a.row_scale;
     auto phase_of = [&](int r) {
         const int row = t.phase_row + r;
         return a.per_l ? ph[(size_t)l * a.N + row] : ph[(size_t)(l & 1) * a.N + phase_entry(l, row, a.N)];
@@ -575,6 +581,11 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
             const double s = re * w.x - im * w.y;
             im = re * w.y + im * w.x;
             re = s;
+        }
+        if (rs) {
+            const double f = rs[t.phase_row + r];
+            re *= f;
+            im *= f;
         }
         double* o = const_cast<double*>(out.at(j, r));
         *o = re;
@@ -588,6 +599,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
             const double2 w = phase_of(r);
             v = j ? o * w.y + v * w.x : v * w.x - o * w.y;
         }
+        if (rs) v *= rs[t.phase_row + r];
         if (j < nline) *const_cast<double*>(out.at(j, r)) = v;
     } else {
 #pragma unroll
@@ -611,7 +623,7 @@ int launch(MmArgs a, const GroupTable& g, cudaStream_t st) {
         a.comp0[0] = a.unit0[0][0] = a.unit0[1][0] = a.unit0[2][0] = 0;
         for (int gi = g.ngroups - 1; gi >= 0; --gi) {
             const int nl = g.line0[gi + 1] - g.line0[gi], l = g.l[gi], lt = (nl + NL - 1) / NL, n = a.npos;
-            if ((nl <= NARROW_MAX) != (NL == 2)) continue;
+            if ((nl <= a.narrow_max) != (NL == 2)) continue;
             const int mtiles = (l + 15) / 16;
             if (a.kind == kMoments && mtiles == 0) continue;
             a.gidx[n] = gi;
@@ -641,7 +653,10 @@ int launch(MmArgs a, const GroupTable& g, cudaStream_t st) {
     return DSBT_OK;
 }
 
-int launch_both(const MmArgs& a, const GroupTable& g, cudaStream_t st) {
+int launch_both(MmArgs a, const GroupTable& g, cudaStream_t st) {
+    int wide = 0;   // CTAs of the wide form at 64 rows each
+    for (int i = 0; i < g.ngroups; ++i) wide += (g.line0[i + 1] - g.line0[i] + 15) / 16 * (a.N / 64);
+    a.narrow_max = wide <= kSMs / 2 ? 16 : 4;
     int rc = launch<16>(a, g, st);
     if (rc == DSBT_OK) rc = launch<2>(a, g, st);
     return rc;
@@ -653,7 +668,7 @@ int launch_both(const MmArgs& a, const GroupTable& g, cudaStream_t st) {
 // line of 256 points (N = 256, l <= 9) to 2048 lines of 2048, at errors against
 // 64-bit references that are equal or smaller.
 int contract_f64(const dsbt_plan* p, const GroupTable& g, int dir, const double* in, int in_cplx, double* out,
-                 int out_cplx, const double2* phase, cudaStream_t st, double* fast_scratch) {
+                 int out_cplx, const double2* phase, cudaStream_t st, double* fast_scratch, const double* row_scale) {
     if (!p->T64) {
         set_error("FP64 path needs a plan built with DSBT_PLAN_FP64");
         return DSBT_ERR_UNSUPPORTED;
@@ -669,6 +684,7 @@ int contract_f64(const dsbt_plan* p, const GroupTable& g, int dir, const double*
     a.in = in;
     a.out = out;
     a.phase = phase;
+    a.row_scale = row_scale;
     a.N = p->N;
     a.R = g.total_lines;
     a.dir = dir;

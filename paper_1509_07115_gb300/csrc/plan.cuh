@@ -90,6 +90,10 @@ int grouped_device_call(int which, const dsbt_plan* p, const int* counts, int dt
 enum : int { kKineticReady = 3 };
 int kinetic_phase_fill(const dsbt_plan* p, void* ws, int total_channels, double tau, cudaStream_t st);
 const double2* kinetic_phase_table(const dsbt_plan* p, void* ws, int total_channels);
+// out = F^T T^T diag(row_scale) T F in of `nchan` real FP64 channels of one l (b: scratch
+// for the coefficients; workspace of a DSBT_F64 call; out may be in).
+int real_step(const dsbt_plan* p, int l, int nchan, const double* in, double* b, double* out, const double* row_scale,
+              void* ws, size_t ws_b, cudaStream_t st);
 
 // ---- plan build (plan.cu)
 int plan_build_factors(dsbt_plan* p, cudaStream_t st);
@@ -138,10 +142,11 @@ int dct_inverse_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
 // group is part s of its channel j); 0: planar lines [line][N].
 // dir = +1: out = T_l in (forward), dir = -1: out = T_l^T in (inverse).
 // phase: optional complex phase per coefficient applied to the result (kinetic
-// step), indexed [parity][N] as double2; nullptr for none.
+// step), indexed [parity][N] as double2; nullptr for none.  row_scale: an optional
+// real factor per coefficient [N] (without a phase).
 int contract_f64(const dsbt_plan* p, const GroupTable& g, int dir, const double* in, int in_cplx,
                  double* out, int out_cplx, const double2* phase, cudaStream_t st,
-                 double* fast_scratch = nullptr);
+                 double* fast_scratch = nullptr, const double* row_scale = nullptr);
 // DSBT_PLAN_FAST64 (fast64.cu); fast_scratch: its moments, fast_scratch_bytes of
 // the call's lines, or nullptr for the dense factors
 bool fast_supported(int N);
