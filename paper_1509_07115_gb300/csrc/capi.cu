@@ -7,6 +7,8 @@
 //                                epilogue -> T_l^T -> F_l^T -> out
 #include <math.h>
 
+#include <algorithm>
+
 #include "plan.cuh"
 
 namespace dsbt {
@@ -42,37 +44,62 @@ __global__ void k_split_lines_c(const float2* __restrict__ in, float* __restrict
 // channel (N values, or N complex values = two lines) computes ||psi||, picks
 // 2^e with ||2^e psi|| in [2^12, 2^13) and writes hi = fp16(2^e x),
 // lo = fp16(2^e x - hi) to the channel's planar lines and 2^-e to scale[line].
-__global__ void k_split_f16(const float* __restrict__ in, int cplx, int N, __half* __restrict__ hi,
-                            __half* __restrict__ lo, float* __restrict__ scale) {
+// HBM-bound when it streams: the channel is read once, 16 bytes a load where the
+// caller's alignment allows (VEC), and held in registers between the norm and the
+// stores (reading it twice in 4-byte loads took 30 us for 1271 real channels of 6400
+// points; now 23 us).
+constexpr int kSplitThreads = 256, kSplitChunks = 16;   // at most: chunks of 4 floats, 16384 floats (complex N = 8192)
+
+template <bool CPLX, bool VEC>
+__global__ void __launch_bounds__(kSplitThreads) k_split_f16(const float* __restrict__ in, int N, __half* __restrict__ hi,
+                                                             __half* __restrict__ lo, float* __restrict__ scale) {
     const long long c = blockIdx.x;
-    const int per = cplx ? 2 : 1;
-    const float* x = in + c * (long long)N * per;
+    const int n4 = N * (CPLX ? 2 : 1) / 4;
+    const float* x = in + c * (long long)n4 * 4;
+    float4 v[kSplitChunks];
     float part = 0.f;
-    for (int i = threadIdx.x; i < N * per; i += blockDim.x) part += x[i] * x[i];
+#pragma unroll
+    for (int q = 0; q < kSplitChunks; ++q) {
+        const int i = threadIdx.x + q * blockDim.x;
+        if (i < n4) {
+            if (VEC) v[q] = reinterpret_cast<const float4*>(x)[i];
+            else v[q] = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+            part += (v[q].x * v[q].x + v[q].y * v[q].y) + (v[q].z * v[q].z + v[q].w * v[q].w);
+        }
+    }
     __shared__ float red[32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
+    float sum = 0.f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) red[0] = v;
-    }
-    __syncthreads();
-    const float nrm = sqrtf(red[0]);
+    for (int w = 0; w < kSplitThreads / 32; ++w)
+        if (w < (int)(blockDim.x >> 5)) sum += red[w];
+    const float nrm = sqrtf(sum);
     const int e = (nrm > 0.f && isfinite(nrm)) ? 12 - ilogbf(nrm) : 0;
     const float fs = ldexpf(1.f, e);
-    const long long line = c * per;
-    if (threadIdx.x < per) scale[line + threadIdx.x] = ldexpf(1.f, -e);
-    for (int i = threadIdx.x; i < N * per; i += blockDim.x) {
-        const int part_ = cplx ? (i & 1) : 0, n = cplx ? (i >> 1) : i;
-        const float v = x[i] * fs;
-        const __half h = __float2half_rn(v);
-        const size_t o = (size_t)(line + part_) * N + n;
-        hi[o] = h;
-        lo[o] = __float2half_rn(v - __half2float(h));
+    const long long line = c * (CPLX ? 2 : 1);
+    if (threadIdx.x < (CPLX ? 2 : 1)) scale[line + threadIdx.x] = ldexpf(1.f, -e);
+    auto pair = [&](size_t at, float a, float b) {   // two consecutive points of a line
+        const float2 f = make_float2(a * fs, b * fs);
+        const __half2 h = __float22half2_rn(f);
+        *reinterpret_cast<__half2*>(hi + at) = h;
+        *reinterpret_cast<__half2*>(lo + at) = __float22half2_rn(make_float2(f.x - __low2float(h), f.y - __high2float(h)));
+    };
+#pragma unroll
+    for (int q = 0; q < kSplitChunks; ++q) {
+        const int i = threadIdx.x + q * blockDim.x;
+        if (i >= n4) break;
+        if (CPLX) {
+            const size_t at = (size_t)line * N + 2 * i;
+            pair(at, v[q].x, v[q].z);
+            pair(at + N, v[q].y, v[q].w);
+        } else {
+            const size_t at = (size_t)line * N + 4 * i;
+            pair(at, v[q].x, v[q].y);
+            pair(at + 2, v[q].z, v[q].w);
+        }
     }
 }
 
@@ -100,6 +127,9 @@ __global__ void k_phase(double2* ph64, float2* ph32, int N, double dk, double ta
     if (ph64) ph64[i] = make_double2(c, s);
     if (ph32) ph32[i] = make_float2((float)c, (float)s);
 }
+
+// One warp per quarter of an SM: its sines are bound by the FP64 pipe.
+constexpr int kPhaseThreads = 128;
 
 // Rows of the phase table (see k_phase).
 inline int phase_rows(const dsbt_plan* p) { return p->knl ? p->l_max + 1 : 2; }
@@ -268,8 +298,12 @@ int run_inverse(const dsbt_plan* p, const GroupTable& g, int dtype, const void* 
     if (p->ftc) {   // interval scheme on FP16 pairs
         {
             ProfScope ps(kKSplit, st);
-            k_split_f16<<<(unsigned)g.chan0[g.ngroups], 256, 0, st>>>((const float*)in, cplx ? 1 : 0, p->N,
-                                                                       w.h_hi_b, w.h_lo_b, w.scale);
+            const bool vec = ((uintptr_t)in & 15) == 0;   // N is a multiple of 256: every channel starts alike
+            const auto k = cplx ? (vec ? k_split_f16<true, true> : k_split_f16<true, false>)
+                                : (vec ? k_split_f16<false, true> : k_split_f16<false, false>);
+            // four chunks a thread where that leaves a warp, so that short channels fill theirs
+            const int n4 = p->N * (cplx ? 2 : 1) / 4, th = std::min(kSplitThreads, std::max(32, n4 / 4 / 32 * 32));
+            k<<<(unsigned)g.chan0[g.ngroups], th, 0, st>>>((const float*)in, p->N, w.h_hi_b, w.h_lo_b, w.scale);
         }
         DSBT_CUDA_TRY(cudaGetLastError());
         rc = contract_split_fast(p, g, -1, w.h_hi_b, w.h_lo_b, w.scale, kOutPlanarF32, w.planar, nullptr, nullptr,
@@ -297,7 +331,7 @@ int run_inverse(const dsbt_plan* p, const GroupTable& g, int dtype, const void* 
 int fill_phase64(const dsbt_plan* p, const Workspace& w, double tau, cudaStream_t st) {
     ProfScope ps(kKPhase, st);
     const int rows = phase_rows(p);
-    k_phase<<<(rows * p->N + 255) / 256, 256, 0, st>>>(w.ph64, nullptr, p->N, p->dk, tau, p->knl, rows);
+    k_phase<<<(rows * p->N + kPhaseThreads - 1) / kPhaseThreads, kPhaseThreads, 0, st>>>(w.ph64, nullptr, p->N, p->dk, tau, p->knl, rows);
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -320,7 +354,7 @@ int run_kinetic(const dsbt_plan* p, const GroupTable& g, int dtype, double tau, 
     {
         ProfScope ps(kKPhase, st);
         const int rows = phase_rows(p);
-        k_phase<<<(rows * N + 255) / 256, 256, 0, st>>>(nullptr, w.ph32, N, p->dk, tau, p->knl, rows);
+        k_phase<<<(rows * N + kPhaseThreads - 1) / kPhaseThreads, kPhaseThreads, 0, st>>>(nullptr, w.ph32, N, p->dk, tau, p->knl, rows);
     }
     DSBT_CUDA_TRY(cudaGetLastError());
     if (p->ftc) {   // interval scheme on FP16 pairs; the lines stay scaled until the last contraction
