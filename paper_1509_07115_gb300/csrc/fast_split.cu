@@ -72,8 +72,12 @@ using namespace tc;
 constexpr int BM = 128;
 constexpr int BK = 64;                             // K elements per block: one 128-byte swizzle row of FP16
 constexpr int BN_MAX = 256;
-constexpr int BBOX = 256;                          // rows per B TMA box (one box per operand half; 64 and 128: 1 % slower)
-constexpr int STAGES = 2;
+// Rows of a B TMA box: a full column tile of 256 lines takes one box per operand half
+// (64- and 128-row boxes: 1 % slower there), any other as many 64-row boxes as hold
+// its lines: a group of 2 .. 126 lines loaded 256 rows with the large box, which bound
+// the launch by its L2 reads (N = 2048, l < 32 all m: 72 -> 57 us a direction with
+// the smaller tiles below).
+constexpr int BBOX = 256, BBOX_S = 64;
 // K blocks per chunk.  The tensor cores accumulate with truncation, and all
 // three split products of a chunk go into one buffer, so the chunk is one K
 // block: the round-trip error at N = 4096, l <= 63 is then 5.6e-7, the dense
@@ -81,14 +85,28 @@ constexpr int STAGES = 2;
 // dense kernel, leaves no TMEM columns for a second buffer).
 constexpr int KC = 1;
 constexpr int EPI_WARPS = 8;                       // two per TMEM lane quarter
-constexpr int WC = BN_MAX * 4 / EPI_WARPS;         // accumulator columns per epilogue warp
 constexpr int QS = 4;                              // tile-queue slots
+// The next tile is fetched when the producer comes to its tile's AHEAD-th last K
+// block: later than that costs the fetch's latency, earlier takes tiles from SMs that
+// would start them sooner (N = 256, l < 47, 8 channels, both directions: 60 us with 1,
+// 75 with 2 or with no such wait, 64 with the producer fetching tiles itself;
+// 4 is 1 % faster than 1 on 4096 x 64 x 8).
+constexpr int AHEAD = 1;
 constexpr int A_BYTES = BM * BK * 2;               // 16 KiB
-constexpr int B_BYTES = BN_MAX * BK * 2;           // 32 KiB
 constexpr float kFacScale = 16384.f;               // plan factors are stored times 2^14
 constexpr float kFacUnscale = 1.f / 16384.f;
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
-constexpr int NTHREADS = 64 + 32 * EPI_WARPS;
+// Column tile of a launch: 256 lines, or 128 or 64 when every group fits one; the
+// smaller stages buy more of them (192 KB in each case).
+template <int BN_>
+struct TileForm {
+    static constexpr int BN = BN_;
+    static constexpr int B_BYTES = BN * BK * 2;
+    static constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;   // 96, 64, 48 KiB
+    static constexpr int STAGES = BN == 256 ? 2 : (BN == 128 ? 3 : 4);
+    static constexpr int WC = BN * 4 / EPI_WARPS;                   // accumulator columns per epilogue warp
+};
+constexpr int MAX_STAGES = 4;
+constexpr int NTHREADS = 96 + 32 * EPI_WARPS;     // TMA, MMA and scheduler warps
 constexpr int FL = 128;                            // leaf = output row tile
 constexpr int KP = 64;                             // basis functions per interval (>= l_max)
 constexpr int MAX_LEVELS = 6;                      // N / 128 <= 64 (plans have N <= 8192)
@@ -162,6 +180,7 @@ __device__ __forceinline__ int block_start(const FtcSpace& fs, int i, int k) {
 // k whose first tile is <= t (blocks may be empty), found by a search over the
 // positions, then over the position's units; blocks k >= U hold second-kind
 // tiles only.
+template <int BN>
 __device__ __forceinline__ Tile decode(const FtcSpace& fs, const GroupTable& gt, int t) {
     const int tail = fs.acum[fs.npos];   // first-kind tiles of the launch
     int k, na = 0;
@@ -203,9 +222,8 @@ __device__ __forceinline__ Tile decode(const FtcSpace& fs, const GroupTable& gt,
     tl.g = g;
     tl.ct = tl.unit - fs.u0[i];
     tl.wait = tl.mode == fs.omode && fs.ta[i] > 0;   // the unit has first-kind tiles
-    const int nl = gt.line0[g + 1] - gt.line0[g];
-    int left = nl - tl.ct * BN_MAX;
-    if (left > BN_MAX) left = BN_MAX;
+    int left = gt.line0[g + 1] - gt.line0[g] - tl.ct * BN;
+    if (left > BN) left = BN;
     tl.nmma = (left + 15) & ~15;
     return tl;
 }
@@ -264,25 +282,9 @@ struct Segs {
         for (int q = 0; q < n; ++q) c += k1[q] - k0[q];
         return c;
     }
-    __device__ __forceinline__ void at(int i, int& s, int& kb, int& akb) const {
-        for (int q = 0; q < n; ++q) {
-            const int len = k1[q] - k0[q];
-            if (i < len) {
-                s = src[q];
-                kb = k0[q] + i;
-                akb = ak[q] + i;
-                return;
-            }
-            i -= len;
-        }
-        s = 1;
-        kb = 0;
-        akb = 0;
-    }
 };
 
-__device__ __forceinline__ Segs segments(const FtcSpace& fs, int mode, int l, int rt) {
-    Segs sg;
+__device__ __forceinline__ void segments(const FtcSpace& fs, int mode, int l, int rt, Segs& sg) {
     sg.n = 0;
     const int nx = n_extra(l);
     const int nf = (l + BK - 1) / BK;   // far K blocks per slot (basis functions k < l)
@@ -334,28 +336,17 @@ __device__ __forceinline__ Segs segments(const FtcSpace& fs, int mode, int l, in
             }
         }
     }
-    return sg;
 }
 
-// Number of K blocks of a tile (what segments(...).count() gives), without
-// building the list.
-__device__ __forceinline__ int seg_count(const FtcSpace& fs, int mode, int l, int rt) {
-    const int nx = n_extra(l);
-    const int nf = (l + BK - 1) / BK;
-    if (mode == kMoments || mode == kWeights) {
-        int a0, a1, b0 = 0, b1 = 0;
-        aug_range(fs, mode, fs.pair_a[rt], a0, a1);
-        if (fs.pair_b[rt] >= 0) aug_range(fs, mode, fs.pair_b[rt], b0, b1);
-        if (b1 <= b0 || (b0 >= a0 && b1 <= a1)) return a1 - a0;
-        if (a0 >= b0 && a1 <= b1) return b1 - b0;
-        return (a1 - a0) + (b1 - b0);
-    }
-    if (mode == kEval) return rt == 0 ? FL / BK + (nx > 0 ? fs.nright * nf : 0) : __popc(rt) * nf + FL / BK;
-    int c = ((rt > 0 && nx > 0) ? 1 : 0) + FL / BK;
-    for (int j = 0; j < fs.levels; ++j)
-        if (used(fs, j, rt >> j)) c += nf;
-    return c;
-}
+// A tile as the scheduler hands it to the other roles.
+struct TileWork {
+    Tile t;
+    int l, nkb, line0, nl;            // angular momentum, K blocks, first line and lines of the group
+    int chan0;
+    int arow1, arow2;                 // A rows: first slot or diagonal block; second slot or far rows
+    int ra0, ra1, rb0, rb1;           // own K ranges of the two slots (first kind)
+    Segs sg;
+};
 
 struct EpiArgs {
     int mode;              // OutMode of the second kind's output
@@ -374,9 +365,8 @@ __device__ __forceinline__ void split_f16(float v, __half& hi, __half& lo) {
     hi = __float2half_rn(v);
     lo = __float2half_rn(v - __half2float(hi));
 }
-// Barriers, the tile queue and two words after the stages (the launch adds
-// 512 bytes past the 1024-byte alignment of the stages).
-static_assert((2 * STAGES + 4 + 2 * QS + 1) * 8 + QS * sizeof(Tile) + 8 <= 512, "control area");
+// Barriers, the tile queue, two words after the stages.
+constexpr int CONTROL_BYTES = (2 * MAX_STAGES + 4 + 2 * QS + 2) * 8 + QS * sizeof(TileWork) + 8;
 
 // Counter block of a launch (zeroed before it): the tile scheduler, the
 // launch-wide abort word and, per unit, the first-kind epilogue warps done.
@@ -426,6 +416,7 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 // The kernel: roles and bounded waits as in gemm_tf32x3.cu; what differs is
 // where each K block comes from, the two kinds of tiles in one launch and the
 // two alternating accumulator buffers.
+template <int BN_>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constant__ CUtensorMap tmA0_lo,
                const __grid_constant__ CUtensorMap tmA1_hi, const __grid_constant__ CUtensorMap tmA1_lo,
@@ -433,7 +424,11 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                const __grid_constant__ CUtensorMap tmA2_hi, const __grid_constant__ CUtensorMap tmA2_lo,
                const __grid_constant__ CUtensorMap tmB2_hi, const __grid_constant__ CUtensorMap tmB2_lo,
                const __grid_constant__ CUtensorMap tmA3_hi, const __grid_constant__ CUtensorMap tmA3_lo,
+               const __grid_constant__ CUtensorMap tmS1_hi, const __grid_constant__ CUtensorMap tmS1_lo,
+               const __grid_constant__ CUtensorMap tmS2_hi, const __grid_constant__ CUtensorMap tmS2_lo,
                GroupTable gt, FtcSpace fs, int N, EpiArgs ep, unsigned* status, uint32_t spin, int* ctr) {
+    using TF = TileForm<BN_>;
+    constexpr int BN = TF::BN, B_BYTES = TF::B_BYTES, STAGE_BYTES = TF::STAGE_BYTES, STAGES = TF::STAGES, WC = TF::WC;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* stage_base = smem;
@@ -444,7 +439,8 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
     uint64_t* tq_full = acc_empty + 2;
     uint64_t* tq_empty = tq_full + QS;
     uint64_t* drain_bar = tq_empty + QS;    // the MMA issuer's exit drain
-    Tile* tile_q = (Tile*)(drain_bar + 1);   // decoded by the producer for the other roles
+    uint64_t* go_bar = drain_bar + 1;       // the producer nears its tile's end
+    TileWork* tile_q = (TileWork*)(go_bar + 1);   // prepared by the scheduler for the other roles
     uint32_t* tmem_slot = (uint32_t*)(tile_q + QS);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
@@ -462,14 +458,15 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
         }
         for (int q = 0; q < QS; ++q) {
             mbar_init(&tq_full[q], 1);
-            mbar_init(&tq_empty[q], 1 + EPI_WARPS);
+            mbar_init(&tq_empty[q], 2 + EPI_WARPS);
         }
         mbar_init(drain_bar, 1);
+        mbar_init(go_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, 512);
+        tmem_alloc(tmem_slot, 2 * BN);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -491,92 +488,73 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
             int qslot = 0;
             uint32_t qphase = 0;
             while (ok) {
-                if (!mbar_wait(&tq_empty[qslot], qphase ^ 1, abort_flag, status, spin)) { ok = false; break; }
-                const int t = atomicAdd(ctr + kCtrSched, 1);
-                Tile tl;
-                if (t < fs.total) tl = decode(fs, gt, t);
-                else tl.mode = -1;
-                tile_q[qslot] = tl;
-                mbar_arrive(&tq_full[qslot]);
-                if (++qslot == QS) { qslot = 0; qphase ^= 1; }
-                if (tl.mode < 0) break;
-                const bool aug = tl.mode == fs.amode;   // two slots per tile, 64 A rows each
-                const int l = gt.l[tl.g];
-                const Segs sg = segments(fs, tl.mode, l, tl.rt);
-                const int nbox = (tl.nmma + BBOX - 1) / BBOX;
-                const bool pair = aug && fs.pair_b[tl.rt] >= 0;
+                if (!mbar_wait(&tq_full[qslot], qphase, abort_flag, status, spin)) break;
+                const TileWork& w = tile_q[qslot];
+                const int mode = w.t.mode;
+                if (mode < 0) break;
+                const bool aug = mode == fs.amode;   // two slots per tile, 64 A rows each
+                const bool pair = aug && fs.pair_b[w.t.rt] >= 0;
+                const int l = w.l, rt = w.t.rt, nmma = w.t.nmma, unit = w.t.unit, arow1 = w.arow1, arow2 = w.arow2;
+                // one 256-row box, or 64-row boxes up to the tile's last line
+                const bool big = BN == BBOX && nmma > BBOX - BBOX_S;
+                const int box = big ? BBOX : BBOX_S, nbox = (nmma + box - 1) / box;
                 const uint32_t a_bytes = (aug ? 64u : 128u) * BK * 2u;
-                const uint32_t bytes = 2 * a_bytes * (pair ? 2 : 1) + 2 * nbox * BBOX * BK * 2;
-                int arow1, arow2 = 0;
-                int ra0 = 0, ra1 = 0, rb0 = 0, rb1 = 0;   // own K ranges of the two slots
-                if (aug) {
-                    aug_range(fs, tl.mode, fs.pair_a[tl.rt], ra0, ra1);
-                    if (pair) aug_range(fs, tl.mode, fs.pair_b[tl.rt], rb0, rb1);
-                }
-                if (tl.mode == kMoments) {
-                    arow1 = ((l & 1) * fs.nslots_f + fs.pair_a[tl.rt]) * KP;
-                    if (pair) arow2 = ((l & 1) * fs.nslots_f + fs.pair_b[tl.rt]) * KP;
-                } else if (tl.mode == kWeights) {   // compact BT: rows (l, level, k)
-                    int j, i;
-                    slot_ji(fs, fs.pair_a[tl.rt], j, i);
-                    arow1 = (l * fs.levels + j) * KP;
-                    if (pair) {
-                        slot_ji(fs, fs.pair_b[tl.rt], j, i);
-                        arow2 = (l * fs.levels + j) * KP;
-                    }
-                } else {
-                    arow1 = (l * fs.nleaf + tl.rt) * BM;   // diagonal block of leaf rt
-                    arow2 = (tl.mode == kEval ? l : (l & 1)) * N + tl.rt * BM;
-                }
-                const int brow = gt.line0[tl.g] + tl.ct * BN_MAX;
-                const int nkb = sg.count();
-                bool waited = !tl.wait;
-                for (int i = 0; i < nkb; ++i) {
-                    int src, kb, akb;
-                    sg.at(i, src, kb, akb);
+                const uint32_t bytes = 2 * a_bytes * (pair ? 2 : 1) + 2 * nbox * box * BK * 2;
+                const int brow = w.line0 + w.t.ct * BN, nseg = w.sg.n;
+                bool waited = !w.t.wait;
+                int left = w.nkb;
+                if (left < AHEAD) mbar_arrive(go_bar);
+                for (int q = 0; q < nseg && ok; ++q) {
+                    const int src = w.sg.src[q], k0 = w.sg.k0[q], k1 = w.sg.k1[q], ak = w.sg.ak[q] - k0;
                     if (src == 2 && !waited) {
-                        if (!wait_unit(ctr + kCtrUnits + tl.unit, unit_target, ctr + kCtrAbort, abort_flag, status,
-                                       spin)) { ok = false; break; }
+                        if (!wait_unit(ctr + kCtrUnits + unit, unit_target, ctr + kCtrAbort, abort_flag, status, spin)) {
+                            ok = false;
+                            break;
+                        }
                         waited = true;
                     }
-                    if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, status, spin)) { ok = false; break; }
-                    unsigned char* sb = stage_base + stage * STAGE_BYTES;
-                    mbar_expect_tx(&full[stage], bytes);
-                    led.arm(stage, phase);
                     const CUtensorMap* ah = aug ? &tmA0_hi : (src == 1 ? &tmA1_hi : (src == 2 ? &tmA2_hi : &tmA3_hi));
                     const CUtensorMap* al = aug ? &tmA0_lo : (src == 1 ? &tmA1_lo : (src == 2 ? &tmA2_lo : &tmA3_lo));
-                    const CUtensorMap* bh = src == 2 ? &tmB2_hi : &tmB1_hi;
-                    const CUtensorMap* bl = src == 2 ? &tmB2_lo : &tmB1_lo;
-                    if (aug) {   // slot a -> A rows 0..63, slot b -> rows 64..127
-                        // a slot's rows are loaded only on its own K range: elsewhere
-                        // (the other slot of a disjoint pair) the load starts past the
-                        // table's last row and the copy fills zeros
-                        const int ya = (kb >= ra0 && kb < ra1) ? arow1 : fs.a_oob;
-                        tma_load_2d(sb, ah, &full[stage], kb * BK, ya);
-                        tma_load_2d(sb + A_BYTES, al, &full[stage], kb * BK, ya);
-                        if (pair) {
-                            const int yb = (kb >= rb0 && kb < rb1) ? arow2 : fs.a_oob;
-                            tma_load_2d(sb + KP * 128, ah, &full[stage], kb * BK, yb);
-                            tma_load_2d(sb + A_BYTES + KP * 128, al, &full[stage], kb * BK, yb);
-                        }
-                    } else {
-                        // near: K block akb of the leaf's diagonal block; far: slot
-                        // akb of the compact B table (forward) or augmented column
-                        // kb of QA (adjoint); completion: T_l rows 0..63 of the leaf's
-                        // columns
-                        const int arow = src == 1 ? arow1 : (src == 2 ? arow2 : l * N + tl.rt * BM);
-                        tma_load_2d(sb, ah, &full[stage], akb * BK, arow);
-                        tma_load_2d(sb + A_BYTES, al, &full[stage], akb * BK, arow);
-                    }
+                    const CUtensorMap* bh = big ? (src == 2 ? &tmB2_hi : &tmB1_hi) : (src == 2 ? &tmS2_hi : &tmS1_hi);
+                    const CUtensorMap* bl = big ? (src == 2 ? &tmB2_lo : &tmB1_lo) : (src == 2 ? &tmS2_lo : &tmS1_lo);
+                    // near: K block of the leaf's diagonal block; far: slot of the compact B
+                    // table (forward) or augmented column of QA (adjoint); completion: T_l
+                    // rows 0..63 of the leaf's columns
+                    const int arow = src == 1 ? arow1 : (src == 2 ? arow2 : l * N + rt * BM);
                     const uint64_t pol = (!aug && src == 1) ? pol_last : pol_keep;
-                    for (int b = 0; b < nbox; ++b) {
-                        tma_load_2d_hint(sb + 2 * A_BYTES + b * BBOX * 128, bh, &full[stage], kb * BK,
-                                         brow + b * BBOX, pol);
-                        tma_load_2d_hint(sb + 2 * A_BYTES + B_BYTES + b * BBOX * 128, bl, &full[stage],
-                                         kb * BK, brow + b * BBOX, pol);
+                    for (int kb = k0; kb < k1; ++kb) {
+                        if (left-- == AHEAD) mbar_arrive(go_bar);
+                        if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, status, spin)) { ok = false; break; }
+                        unsigned char* sb = stage_base + stage * STAGE_BYTES;
+                        mbar_expect_tx(&full[stage], bytes);
+                        led.arm(stage, phase);
+                        if (aug) {   // slot a -> A rows 0..63, slot b -> rows 64..127
+                            // a slot's rows are loaded only on its own K range: elsewhere
+                            // (the other slot of a disjoint pair) the load starts past the
+                            // table's last row and the copy fills zeros
+                            const int ya = (kb >= w.ra0 && kb < w.ra1) ? arow1 : fs.a_oob;
+                            tma_load_2d(sb, ah, &full[stage], kb * BK, ya);
+                            tma_load_2d(sb + A_BYTES, al, &full[stage], kb * BK, ya);
+                            if (pair) {
+                                const int yb = (kb >= w.rb0 && kb < w.rb1) ? arow2 : fs.a_oob;
+                                tma_load_2d(sb + KP * 128, ah, &full[stage], kb * BK, yb);
+                                tma_load_2d(sb + A_BYTES + KP * 128, al, &full[stage], kb * BK, yb);
+                            }
+                        } else {
+                            tma_load_2d(sb, ah, &full[stage], (ak + kb) * BK, arow);
+                            tma_load_2d(sb + A_BYTES, al, &full[stage], (ak + kb) * BK, arow);
+                        }
+                        for (int b = 0; b < nbox; ++b) {
+                            tma_load_2d_hint(sb + 2 * A_BYTES + b * box * 128, bh, &full[stage], kb * BK,
+                                             brow + b * box, pol);
+                            tma_load_2d_hint(sb + 2 * A_BYTES + B_BYTES + b * box * 128, bl, &full[stage],
+                                             kb * BK, brow + b * box, pol);
+                        }
+                        if (++stage == STAGES) { stage = 0; phase ^= 1; }
                     }
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
                 }
+                mbar_arrive(&tq_empty[qslot]);
+                if (++qslot == QS) { qslot = 0; qphase ^= 1; }
             }
             led.drain(full, STAGES, status);   // copies still in flight after an abort
         }
@@ -591,13 +569,11 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
             uint32_t qphase = 0;
             while (ok) {
                 if (!mbar_wait(&tq_full[qslot], qphase, abort_flag, status, spin)) break;
-                const Tile tl = tile_q[qslot];
+                const int mode = tile_q[qslot].t.mode, nkb = tile_q[qslot].nkb;
+                const uint32_t idesc = idesc_f16(BM, tile_q[qslot].t.nmma);
                 mbar_arrive(&tq_empty[qslot]);
                 if (++qslot == QS) { qslot = 0; qphase ^= 1; }
-                if (tl.mode < 0) break;
-                const int l = gt.l[tl.g];
-                const int nkb = seg_count(fs, tl.mode, l, tl.rt);
-                const uint32_t idesc = idesc_f16(BM, tl.nmma);
+                if (mode < 0) break;
                 for (int c0 = 0; c0 < nkb && ok; c0 += fs.kc) {
                     const int c1 = min(nkb, c0 + fs.kc);
                     const int buf = gch & 1;
@@ -605,7 +581,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                     // buffer may still be draining while these MMAs run
                     if (!mbar_wait(&acc_empty[buf], ((gch >> 1) & 1) ^ 1, abort_flag, status, spin)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t d = tmem_base + (uint32_t)buf * 256;
+                    const uint32_t d = tmem_base + (uint32_t)buf * BN;
                     uint32_t accf = 0;
                     for (int i = c0; i < c1; ++i) {
                         if (!mbar_wait(&full[stage], phase, abort_flag, status, spin)) { ok = false; break; }
@@ -635,6 +611,59 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
             mma_drain(drain_bar, status);   // every MMA issued has finished
         }
         __syncwarp();
+    } else if (warp == 2 + EPI_WARPS) {
+        // ------------------------------------------------ scheduler: fetches the next
+        // tile and prepares it, so that neither the atomic's latency nor the searches
+        // stand between two tiles' loads.  Tiles of few K blocks gain most: N = 2048,
+        // l < 32 all m 57 -> 50 us a direction (the L2 at 20 % before), N = 6400 of
+        // 100 channels 148 -> 136 us, N = 4096, l < 64 x 8 1235 -> 1222 us.
+        if (lane == 0) {
+            int qslot = 0;
+            uint32_t qphase = 0, go = 1;   // the first tile needs no go
+            while (mbar_wait(go_bar, go, abort_flag, status, spin) &&
+                   mbar_wait(&tq_empty[qslot], qphase ^ 1, abort_flag, status, spin)) {
+                go ^= 1;
+                const int t = atomicAdd(ctr + kCtrSched, 1);
+                TileWork& w = tile_q[qslot];
+                if (t >= fs.total) {
+                    w.t.mode = -1;
+                    mbar_arrive(&tq_full[qslot]);
+                    break;
+                }
+                const Tile tl = decode<BN>(fs, gt, t);
+                const bool aug = tl.mode == fs.amode;
+                const int l = gt.l[tl.g];
+                w.t = tl;
+                w.l = l;
+                w.line0 = gt.line0[tl.g];
+                w.nl = gt.line0[tl.g + 1] - w.line0;
+                w.chan0 = gt.chan0[tl.g];
+                segments(fs, tl.mode, l, tl.rt, w.sg);
+                w.nkb = w.sg.count();
+                if (aug) {
+                    const int sa = fs.pair_a[tl.rt], sb = fs.pair_b[tl.rt];
+                    int j, i;
+                    w.rb0 = w.rb1 = 0;
+                    aug_range(fs, tl.mode, sa, w.ra0, w.ra1);
+                    if (sb >= 0) aug_range(fs, tl.mode, sb, w.rb0, w.rb1);
+                    if (tl.mode == kMoments) {
+                        w.arow1 = ((l & 1) * fs.nslots_f + sa) * KP;
+                        w.arow2 = ((l & 1) * fs.nslots_f + sb) * KP;
+                    } else {   // compact BT: rows (l, level, k)
+                        slot_ji(fs, sa, j, i);
+                        w.arow1 = (l * fs.levels + j) * KP;
+                        if (sb >= 0) slot_ji(fs, sb, j, i);
+                        w.arow2 = (l * fs.levels + j) * KP;
+                    }
+                } else {
+                    w.arow1 = (l * fs.nleaf + tl.rt) * BM;   // diagonal block of leaf rt
+                    w.arow2 = (tl.mode == kEval ? l : (l & 1)) * N + tl.rt * BM;
+                }
+                mbar_arrive(&tq_full[qslot]);   // release: this thread wrote the entry
+                if (++qslot == QS) { qslot = 0; qphase ^= 1; }
+            }
+        }
+        __syncwarp();
     } else {
         // ------------------------------------------------ epilogue (EPI_WARPS warps)
         const int ew = warp - 2;
@@ -645,15 +674,14 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
         uint32_t qphase = 0;
         while (true) {
             if (!warp_all(mbar_wait(&tq_full[qslot], qphase, abort_flag, status, spin))) break;
-            const Tile tl = tile_q[qslot];
+            const Tile tl = tile_q[qslot].t;
+            const int l = tile_q[qslot].l, nkb = tile_q[qslot].nkb, nl = tile_q[qslot].nl;
+            const int line0 = tile_q[qslot].line0, chan0 = tile_q[qslot].chan0;
             __syncwarp();
             if (lane == 0) mbar_arrive(&tq_empty[qslot]);
             if (++qslot == QS) { qslot = 0; qphase ^= 1; }
             if (tl.mode < 0) break;
             const bool aug = tl.mode == fs.amode;
-            const int l = gt.l[tl.g];
-            const int nkb = seg_count(fs, tl.mode, l, tl.rt);
-            const int nl = gt.line0[tl.g + 1] - gt.line0[tl.g];
             const int trow = quarter * 32 + lane;                 // TMEM lane = A row of the tile
             int row = tl.rt * BM + trow;
             bool store_row = true;
@@ -662,7 +690,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                 store_row = slot >= 0;
                 row = slot * KP + (trow & (KP - 1));
             }
-            const int cbase = tl.ct * BN_MAX + half * WC;
+            const int cbase = tl.ct * BN + half * WC;
             const int ncols = min(WC, nl - cbase);
             const int nch = (tl.nmma > half * WC) ? ((min(tl.nmma - half * WC, WC) + 31) >> 5) : 0;
             const uint32_t tl_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * WC);
@@ -678,7 +706,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                 for (int ch = 0; ch < WC / 32; ++ch) {
                     if (ch < nch) {
                         float v[32];
-                        tmem_ld32(tl_addr + (uint32_t)buf * 256 + ch * 32, v);
+                        tmem_ld32(tl_addr + (uint32_t)buf * BN + ch * 32, v);
 #pragma unroll
                         for (int j = 0; j < 32; ++j) acc[ch * 32 + j] += v[j];
                     }
@@ -695,7 +723,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                     const int S = ep.astride;
                     __half* o0 = ep.aug0;
                     __half* o1 = ep.aug1;
-                    const size_t line_base = (size_t)gt.line0[tl.g] + cbase;
+                    const size_t line_base = (size_t)line0 + cbase;
 #pragma unroll
                     for (int j = 0; j < WC; ++j) {
                         if (j < ncols) {
@@ -719,7 +747,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
             if (!do_store) continue;
             float2 ph = make_float2(1.f, 0.f);
             if (ep.phase) ph = ep.per_l ? ep.phase[(size_t)l * N + row] : ep.phase[(size_t)(l & 1) * N + phase_entry(l, row, N)];
-            const size_t line_base = (size_t)gt.line0[tl.g] + cbase;
+            const size_t line_base = (size_t)line0 + cbase;
             if (ep.mode == kOutPlanarF32) {
                 float* o = reinterpret_cast<float*>(ep.out0);
 #pragma unroll
@@ -727,7 +755,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                     if (j < ncols) o[(line_base + j) * N + row] = acc[j] * (ep.scale[line_base + j] * kFacUnscale);
             } else if (ep.mode == kOutUserC64) {
                 float2* o = reinterpret_cast<float2*>(ep.out0);
-                const size_t chan_base = (size_t)gt.chan0[tl.g] + (cbase >> 1);
+                const size_t chan_base = (size_t)chan0 + (cbase >> 1);
                 if (gt.uoff) {   // channels gathered by offset (uneven batch)
 #pragma unroll
                     for (int j = 0; j < WC; j += 2)
@@ -745,7 +773,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
                 }
             } else if (ep.mode == kOutUserF32) {
                 float* o = reinterpret_cast<float*>(ep.out0);
-                const size_t chan_base = (size_t)gt.chan0[tl.g] + cbase;
+                const size_t chan_base = (size_t)chan0 + cbase;
 #pragma unroll
                 for (int j = 0; j < WC; ++j)
                     if (j < ncols) {
@@ -779,7 +807,7 @@ k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constan
     if (threadIdx.x == 0 && *abort_flag) atomicExch(ctr + kCtrAbort, 1);   // waiters elsewhere give up
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc(tmem_base, 2 * BN);
     }
 }
 
@@ -1155,10 +1183,12 @@ namespace {
 
 // One launch over the groups (largest l first): the first kind (MOMENTS or
 // WEIGHTS) and the second (EVAL or LEAFOUT) of every unit, interleaved.
+template <int BN>
 int launch_fused(const dsbt_plan* p, const GroupTable& g, int dir, const CUtensorMap& a0h, const CUtensorMap& a0l,
                  const CUtensorMap& a1h, const CUtensorMap& a1l, const CUtensorMap& b1h, const CUtensorMap& b1l,
                  const CUtensorMap& a2h, const CUtensorMap& a2l, const CUtensorMap& b2h, const CUtensorMap& b2l,
-                 const CUtensorMap& a3h, const CUtensorMap& a3l, const EpiArgs& ep, int* ctr, size_t lines,
+                 const CUtensorMap& a3h, const CUtensorMap& a3l, const CUtensorMap& s1h, const CUtensorMap& s1l,
+                 const CUtensorMap& s2h, const CUtensorMap& s2l, const EpiArgs& ep, int* ctr, size_t lines,
                  cudaStream_t st) {
     const FtcData* f = p->ftc;
     FtcSpace fs = f->base;
@@ -1181,7 +1211,7 @@ int launch_fused(const dsbt_plan* p, const GroupTable& g, int dir, const CUtenso
         const int gi = g.ngroups - 1 - i;
         const int nl = g.line0[gi + 1] - g.line0[gi];
         fs.order[i] = gi;
-        const int ct = (nl + BN_MAX - 1) / BN_MAX;
+        const int ct = (nl + BN - 1) / BN;
         fs.ta[i] = g.l[gi] == 0 ? 0 : fs.npairs;   // T_0 has no entries left of its diagonal
         fs.u0[i + 1] = fs.u0[i] + ct;
         fs.acum[i + 1] = fs.acum[i] + ct * fs.ta[i];
@@ -1194,17 +1224,14 @@ int launch_fused(const dsbt_plan* p, const GroupTable& g, int dir, const CUtenso
     }
     fs.lag = std::max(1, std::min(f->lag, fs.units));
     fs.total = fs.acum[g.ngroups] + fs.units * fs.RT;
-    const size_t smem = (size_t)STAGES * STAGE_BYTES + 1024 + 512;
-    int rc = ensure_smem((const void*)k_contract_ftc, smem);
+    const size_t smem = (size_t)TileForm<BN>::STAGES * TileForm<BN>::STAGE_BYTES + 1024 + CONTROL_BYTES;
+    int rc = ensure_smem((const void*)k_contract_ftc<BN>, smem);
     if (rc) return rc;
-    int dev = 0, nsm = 0;
-    DSBT_CUDA_TRY(cudaGetDevice(&dev));
-    DSBT_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int grid = fs.total < nsm ? fs.total : nsm;
+    const int grid = fs.total < kSMs ? fs.total : kSMs;
     DSBT_CUDA_TRY(cudaMemsetAsync(ctr, 0, sizeof(int) * (kCtrUnits + fs.units), st));
     ProfScope ps(kKContractTF32, st);
-    k_contract_ftc<<<grid, NTHREADS, smem, st>>>(a0h, a0l, a1h, a1l, b1h, b1l, a2h, a2l, b2h, b2l, a3h, a3l, g, fs,
-                                                 p->N, ep, p->status, p->spin_limit, ctr);
+    k_contract_ftc<BN><<<grid, NTHREADS, smem, st>>>(a0h, a0l, a1h, a1l, b1h, b1l, a2h, a2l, b2h, b2l, a3h, a3l, s1h,
+                                                     s1l, s2h, s2l, g, fs, p->N, ep, p->status, p->spin_limit, ctr);
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -1233,18 +1260,25 @@ int contract_split_fast(const dsbt_plan* p, const GroupTable& g, int dir, const 
     __half* aug_hi = reinterpret_cast<__half*>(scratch);
     __half* aug_lo = aug_hi + R * NA;
     int* ctr = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(scratch) + ftc_aug_bytes(p, R));
-    CUtensorMap in_h, in_l, aug_h, aug_l;
+    CUtensorMap in_h, in_l, aug_h, aug_l, ins_h, ins_l, augs_h, augs_l;   // 256-row boxes, and 64-row ones
     int rc = encode_tmap_f16_sw128(&in_h, in_hi, R, N, BBOX, BK);
     if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&in_l, in_lo, R, N, BBOX, BK);
     if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&aug_h, aug_hi, R, NA, BBOX, BK);
     if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&aug_l, aug_lo, R, NA, BBOX, BK);
+    if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&ins_h, in_hi, R, N, BBOX_S, BK);
+    if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&ins_l, in_lo, R, N, BBOX_S, BK);
+    if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&augs_h, aug_hi, R, NA, BBOX_S, BK);
+    if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&augs_l, aug_lo, R, NA, BBOX_S, BK);
     if (rc != DSBT_OK) return rc;
     const EpiArgs ep{out_mode, out0, out1, phase, p->knl != nullptr, scale, aug_hi, aug_lo, NA};
+    int most = 0;   // lines of the largest group
+    for (int i = 0; i < g.ngroups; ++i) most = std::max(most, g.line0[i + 1] - g.line0[i]);
+    const auto launch = most <= 64 ? launch_fused<64> : (most <= 128 ? launch_fused<128> : launch_fused<BN_MAX>);
     if (dir > 0)
-        return launch_fused(p, g, dir, f->tm_qT_hi, f->tm_qT_lo, f->tm_D_hi, f->tm_D_lo, in_h, in_l, f->tm_bA_hi,
-                            f->tm_bA_lo, aug_h, aug_l, f->tm_D_hi, f->tm_D_lo, ep, ctr, R, st);
-    return launch_fused(p, g, dir, f->tm_bT_hi, f->tm_bT_lo, f->tm_Dt_hi, f->tm_Dt_lo, in_h, in_l, f->tm_qA_hi,
-                        f->tm_qA_lo, aug_h, aug_l, f->tm_C_hi, f->tm_C_lo, ep, ctr, R, st);
+        return launch(p, g, dir, f->tm_qT_hi, f->tm_qT_lo, f->tm_D_hi, f->tm_D_lo, in_h, in_l, f->tm_bA_hi, f->tm_bA_lo,
+                      aug_h, aug_l, f->tm_D_hi, f->tm_D_lo, ins_h, ins_l, augs_h, augs_l, ep, ctr, R, st);
+    return launch(p, g, dir, f->tm_bT_hi, f->tm_bT_lo, f->tm_Dt_hi, f->tm_Dt_lo, in_h, in_l, f->tm_qA_hi, f->tm_qA_lo,
+                  aug_h, aug_l, f->tm_C_hi, f->tm_C_lo, ins_h, ins_l, augs_h, augs_l, ep, ctr, R, st);
 }
 
 }  // namespace dsbt
