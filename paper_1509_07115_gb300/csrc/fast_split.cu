@@ -26,7 +26,7 @@
 //
 // Every step is then the contraction of gemm_tf32x3.cu with other operands and
 // K ranges.  Tiles are short (4-16 K blocks), so the TMEM accumulator is split
-// into two 256-column buffers used by alternate chunks of KC K blocks (all three
+// into two buffers of a tile's columns used by alternate chunks of KC K blocks (all three
 // split products of a chunk into one buffer): the MMAs of the next chunk, also
 // across tiles, run while the epilogue drains the previous one.
 //   forward   MOMENTS  M[line][(s,k)]  = sum_t QT[(s,k)][t] f[line][t]          (t in interval s)
@@ -95,8 +95,8 @@ constexpr int AHEAD = 1;
 constexpr int A_BYTES = BM * BK * 2;               // 16 KiB
 constexpr float kFacScale = 16384.f;               // plan factors are stored times 2^14
 constexpr float kFacUnscale = 1.f / 16384.f;
-// Column tile of a launch: 256 lines, or 128 or 64 when every group fits one; the
-// smaller stages buy more of them (192 KB in each case).
+// Column tile of a launch: 256, 128 or 64 lines (rule in contract_split_fast); the smaller
+// stages buy more of them (192 KB in each case).
 template <int BN_>
 struct TileForm {
     static constexpr int BN = BN_;
@@ -1271,9 +1271,19 @@ int contract_split_fast(const dsbt_plan* p, const GroupTable& g, int dir, const 
     if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&augs_l, aug_lo, R, NA, BBOX_S, BK);
     if (rc != DSBT_OK) return rc;
     const EpiArgs ep{out_mode, out0, out1, phase, p->knl != nullptr, scale, aug_hi, aug_lo, NA};
-    int most = 0;   // lines of the largest group
-    for (int i = 0; i < g.ngroups; ++i) most = std::max(most, g.line0[i + 1] - g.line0[i]);
-    const auto launch = most <= 64 ? launch_fused<64> : (most <= 128 ? launch_fused<128> : launch_fused<BN_MAX>);
+    // Column tiles: 64 lines when every group fits one; 128 unless they are more than
+    // 7/5 of the 256-line tiles (three stages instead of two against more reads of the
+    // factors; complex lines of all m, 256 -> 128: N = 2048, l <= 33 with 34 -> 36 tiles
+    // a row 80 -> 69 us, l <= 45 with 46 -> 60 tiles 110 -> 103 us, l <= 40 x 2 with
+    // 50 -> 75 tiles 133 us both).
+    int most = 0, t256 = 0, t128 = 0;
+    for (int i = 0; i < g.ngroups; ++i) {
+        const int nl = g.line0[i + 1] - g.line0[i];
+        most = std::max(most, nl);
+        t256 += (nl + 255) / 256;
+        t128 += (nl + 127) / 128;
+    }
+    const auto launch = most <= 64 ? launch_fused<64> : (5 * t128 <= 7 * t256 ? launch_fused<128> : launch_fused<BN_MAX>);
     if (dir > 0)
         return launch(p, g, dir, f->tm_qT_hi, f->tm_qT_lo, f->tm_D_hi, f->tm_D_lo, in_h, in_l, f->tm_bA_hi, f->tm_bA_lo,
                       aug_h, aug_l, f->tm_D_hi, f->tm_D_lo, ins_h, ins_l, augs_h, augs_l, ep, ctr, R, st);
