@@ -9,7 +9,7 @@
 // (A_lo B_lo ~ 2^-22 dropped), which keeps about 2^-21 relative accuracy per
 // product while every MMA runs at TF32 tensor rate.
 //
-// Tiles: 128 output rows (TMEM lanes) x up to 256 real lines (TMEM columns);
+// Tiles: 128 output rows (TMEM lanes) x up to 256 or 128 real lines (TMEM columns);
 // K in blocks of 32 (one 128-byte swizzle row of FP32).  A tile never reads the
 // zero upper triangle of T_l: forward row tile [r0, r0+128) reads K < r0+128
 // (all K when it holds completion rows); inverse tile reads the completion rows
@@ -17,7 +17,7 @@
 //
 // CTA roles (320 threads, one CTA per SM, persistent over a cost-ordered tile
 // list): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, warps 2-9 =
-// epilogue (two warps per TMEM lane quarter, 128 columns each: drain the main
+// epilogue (two warps per TMEM lane quarter, half the columns each: drain the main
 // accumulator every KC K-blocks into FP32 registers, then the optional kinetic
 // phase + TF32 split, then global stores, which overlap the next tile's MMAs).
 // Every mbarrier wait is bounded: on expiry the kernel records kStatusTimeout
@@ -35,13 +35,19 @@ constexpr int BM = 128;
 constexpr int BK = 32;
 constexpr int BN_MAX = 256;
 constexpr int BBOX = 64;                           // rows per B TMA box
-constexpr int STAGES = 2;
 constexpr int KC = 4;                              // K blocks per main-accumulator chunk
 constexpr int EPI_WARPS = 8;
 constexpr int QS = 4;                              // tile-queue slots (scheduler -> MMA, epilogue)
 constexpr int A_BYTES = BM * BK * 4;               // 16 KiB
-constexpr int B_BYTES = BN_MAX * BK * 4;           // 32 KiB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
+// Column tile of a launch: 256 or 128 lines, with as many stages as 192 KB hold.
+template <int BN_>
+struct TileForm {
+    static constexpr int BN = BN_;
+    static constexpr int B_BYTES = BN * BK * 4;                     // 32, 16 KiB
+    static constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;   // 96, 64 KiB
+    static constexpr int STAGES = BN == 256 ? 2 : 3;
+    static constexpr int WC = BN * 4 / EPI_WARPS;                   // accumulator columns per epilogue warp
+};
 constexpr int NTHREADS = 64 + 32 * EPI_WARPS;
 // B lines are re-read by every row tile of their group: keep them in L2.
 #ifndef DSBT_B_EVICT_LAST
@@ -68,6 +74,7 @@ struct Tile {
     int g, rt, ct, nmma;
 };
 
+template <int BN>
 __device__ __forceinline__ Tile decode(const TileSpace& ts, const GroupTable& gt, int dir, int t) {
     Tile tl;
     int i = 0;
@@ -79,8 +86,8 @@ __device__ __forceinline__ Tile decode(const TileSpace& ts, const GroupTable& gt
     tl.ct = local - q * ts.ct[i];
     tl.rt = (dir > 0) ? (q == 0 ? 0 : ts.RT - q) : q;
     const int nl = gt.line0[g + 1] - gt.line0[g];
-    int left = nl - tl.ct * BN_MAX;
-    if (left > BN_MAX) left = BN_MAX;
+    int left = nl - tl.ct * BN;
+    if (left > BN) left = BN;
     tl.nmma = (left + 15) & ~15;
     return tl;
 }
@@ -131,11 +138,14 @@ struct EpiArgs {
 // sum is restarted every KC blocks and the chunk sums are added in FP32 with
 // round-to-nearest in the epilogue's registers; the correction terms are
 // 2^-11 smaller and stay in TMEM for the whole tile.
+template <int BN_>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_constant__ CUtensorMap tmA_lo,
                   const __grid_constant__ CUtensorMap tmB_hi, const __grid_constant__ CUtensorMap tmB_lo,
                   GroupTable gt, TileSpace ts, int N, int dir, EpiArgs ep, unsigned* status,
                   uint32_t spin, int* sched) {
+    using TF = TileForm<BN_>;
+    constexpr int BN = TF::BN, B_BYTES = TF::B_BYTES, STAGE_BYTES = TF::STAGE_BYTES, STAGES = TF::STAGES, WC = TF::WC;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* stage_base = smem;
@@ -199,13 +209,13 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
                 mbar_arrive(&tq_full[qslot]);
                 if (++qslot == QS) { qslot = 0; qphase ^= 1; }
                 if (t < 0) break;
-                const Tile tl = decode(ts, gt, dir, t);
+                const Tile tl = decode<BN>(ts, gt, dir, t);
                 const int l = gt.l[tl.g];
                 const KRange kr = kranges(dir, tl.rt, n_extra(l), ts.KB);
                 const int nbox = (tl.nmma + BBOX - 1) / BBOX;
                 const uint32_t bytes = 2 * A_BYTES + 2 * nbox * BBOX * BK * 4;
                 const int arow = l * N + tl.rt * BM;
-                const int brow = gt.line0[tl.g] + tl.ct * BN_MAX;
+                const int brow = gt.line0[tl.g] + tl.ct * BN;
                 const int nkb = kr.count();
                 for (int i = 0; i < nkb; ++i) {
                     const int kb = kr.at(i);
@@ -249,7 +259,7 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
                 mbar_arrive(&tq_empty[qslot]);
                 if (++qslot == QS) { qslot = 0; qphase ^= 1; }
                 if (t < 0) break;
-                const Tile tl = decode(ts, gt, dir, t);
+                const Tile tl = decode<BN>(ts, gt, dir, t);
                 const int l = gt.l[tl.g];
                 const KRange kr = kranges(dir, tl.rt, n_extra(l), ts.KB);
                 const uint32_t idesc = idesc_tf32(BM, tl.nmma);
@@ -320,7 +330,7 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
         // ------------------------------------------------ epilogue (EPI_WARPS warps)
         const int ew = warp - 2;
         const int quarter = warp & 3;             // TMEM lane quarter this warp may access
-        const int half = ew >> 2;                 // which 128 of the 256 columns
+        const int half = ew >> 2;                 // which half of the columns
         uint32_t mphase = 0;
         int qslot = 0;
         uint32_t qphase = 0;
@@ -331,19 +341,19 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
             if (lane == 0) mbar_arrive(&tq_empty[qslot]);
             if (++qslot == QS) { qslot = 0; qphase ^= 1; }
             if (t < 0) break;
-            const Tile tl = decode(ts, gt, dir, t);
+            const Tile tl = decode<BN>(ts, gt, dir, t);
             const int l = gt.l[tl.g];
             const KRange kr = kranges(dir, tl.rt, n_extra(l), ts.KB);
             const int nkb = kr.count();
             const int nl = gt.line0[tl.g + 1] - gt.line0[tl.g];
             const int row = tl.rt * BM + quarter * 32 + lane;
-            const int cbase = tl.ct * BN_MAX + half * 128;     // first line of this thread's columns
-            const int ncols = min(128, nl - cbase);           // may be <= 0
-            const int nch = (tl.nmma > half * 128) ? ((min(tl.nmma - half * 128, 128) + 31) >> 5) : 0;
-            const uint32_t tl_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 128);
-            float acc[128];
+            const int cbase = tl.ct * BN + half * WC;     // first line of this thread's columns
+            const int ncols = min(WC, nl - cbase);            // may be <= 0
+            const int nch = (tl.nmma > half * WC) ? ((min(tl.nmma - half * WC, WC) + 31) >> 5) : 0;
+            const uint32_t tl_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * WC);
+            float acc[WC];
 #pragma unroll
-            for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+            for (int j = 0; j < WC; ++j) acc[j] = 0.f;
             bool ok = true;
             for (int c0 = 0; c0 < nkb; c0 += KC) {
                 if (!warp_all(mbar_wait(main_full, mphase, abort_flag, status, spin))) { ok = false; break; }
@@ -351,7 +361,7 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
                 tc_fence_after();
                 const bool last = c0 + KC >= nkb;
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
+                for (int ch = 0; ch < WC / 32; ++ch) {
                     if (ch < nch) {
                         float v[32];
                         tmem_ld32(tl_addr + ch * 32, v);
@@ -376,22 +386,22 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
                 float2* o = reinterpret_cast<float2*>(ep.out0);
                 const size_t chan_base = (size_t)gt.chan0[tl.g] + (cbase >> 1);
 #pragma unroll
-                for (int j = 0; j < 128; j += 2)
+                for (int j = 0; j < WC; j += 2)
                     if (j < ncols) o[(chan_base + (j >> 1)) * N + row] = make_float2(acc[j], acc[j + 1]);
             } else if (ep.mode == kOutUserF32) {
                 const size_t chan_base = (size_t)gt.chan0[tl.g] + cbase;
 #pragma unroll
-                for (int j = 0; j < 128; ++j)
+                for (int j = 0; j < WC; ++j)
                     if (j < ncols) ep.out0[(chan_base + j) * N + row] = acc[j];
             } else if (ep.mode == kOutPlanarF32) {
                 const size_t line_base = (size_t)gt.line0[tl.g] + cbase;
 #pragma unroll
-                for (int j = 0; j < 128; ++j)
+                for (int j = 0; j < WC; ++j)
                     if (j < ncols) ep.out0[(line_base + j) * N + row] = acc[j];
             } else {   // kOutPlanarSplit: complex pairs with optional phase, TF32 split
                 const size_t line_base = (size_t)gt.line0[tl.g] + cbase;
 #pragma unroll
-                for (int j = 0; j < 128; j += 2) {
+                for (int j = 0; j < WC; j += 2) {
                     if (j < ncols) {
                         const float re = acc[j] * ph.x - acc[j + 1] * ph.y;
                         const float im = acc[j] * ph.y + acc[j + 1] * ph.x;
@@ -415,6 +425,40 @@ k_contract_tf32x3(const __grid_constant__ CUtensorMap tmA_hi, const __grid_const
     }
 }
 
+// Column tiles of bn lines over a call's groups.
+int column_tiles(const GroupTable& g, int bn) {
+    int n = 0;
+    for (int i = 0; i < g.ngroups; ++i) n += (g.line0[i + 1] - g.line0[i] + bn - 1) / bn;
+    return n;
+}
+
+template <int BN>
+int launch(const dsbt_plan* p, const GroupTable& g, int dir, const CUtensorMap& tb_hi, const CUtensorMap& tb_lo,
+           const EpiArgs& ep, int* sched, cudaStream_t st) {
+    TileSpace ts;
+    ts.RT = p->N / BM;
+    ts.KB = p->N / BK;
+    ts.t0[0] = 0;
+    for (int i = 0; i < g.ngroups; ++i) {
+        const int gi = g.ngroups - 1 - i;   // largest l first
+        const int nl = g.line0[gi + 1] - g.line0[gi];
+        ts.order[i] = gi;
+        ts.ct[i] = (nl + BN - 1) / BN;
+        ts.t0[i + 1] = ts.t0[i] + ts.RT * ts.ct[i];
+    }
+    ts.total = ts.t0[g.ngroups];
+    const size_t smem = (size_t)TileForm<BN>::STAGES * TileForm<BN>::STAGE_BYTES + 1024 + 256;
+    if (int rc = ensure_smem((const void*)k_contract_tf32x3<BN>, smem)) return rc;
+    const CUtensorMap& ahi = dir > 0 ? p->tm_T_hi : p->tm_Tt_hi;
+    const CUtensorMap& alo = dir > 0 ? p->tm_T_lo : p->tm_Tt_lo;
+    DSBT_CUDA_TRY(cudaMemsetAsync(sched, 0, sizeof(int), st));
+    ProfScope ps(kKContractTF32, st);
+    k_contract_tf32x3<BN><<<ts.total < kSMs ? ts.total : kSMs, NTHREADS, smem, st>>>(
+        ahi, alo, tb_hi, tb_lo, g, ts, p->N, dir, ep, p->status, p->spin_limit, sched);
+    DSBT_CUDA_TRY(cudaGetLastError());
+    return DSBT_OK;
+}
+
 }  // namespace
 
 unsigned tc_default_spin_limit() { return tc::kSpinLimit; }
@@ -427,19 +471,7 @@ int contract_tf32x3(const dsbt_plan* p, const GroupTable& g, int dir, const floa
         return DSBT_ERR_UNSUPPORTED;
     }
     const int N = p->N;
-    TileSpace ts;
-    ts.RT = N / BM;
-    ts.KB = N / BK;
-    ts.t0[0] = 0;
-    for (int i = 0; i < g.ngroups; ++i) {
-        const int gi = g.ngroups - 1 - i;   // largest l first
-        const int nl = g.line0[gi + 1] - g.line0[gi];
-        ts.order[i] = gi;
-        ts.ct[i] = (nl + BN_MAX - 1) / BN_MAX;
-        ts.t0[i + 1] = ts.t0[i] + ts.RT * ts.ct[i];
-    }
-    ts.total = ts.t0[g.ngroups];
-    if (ts.total == 0) return DSBT_OK;
+    if (g.total_lines == 0) return DSBT_OK;
     if (out_mode == kOutPlanarSplit || out_mode == kOutUserC64) {
         for (int i = 0; i < g.ngroups; ++i) {
             if ((g.line0[i] & 1) || ((g.line0[i + 1] - g.line0[i]) & 1)) {
@@ -452,22 +484,16 @@ int contract_tf32x3(const dsbt_plan* p, const GroupTable& g, int dir, const floa
     int rc = encode_tmap_f32_sw128(&tb_hi, in_hi, (uint64_t)g.total_lines, N, BBOX, BK);
     if (rc == DSBT_OK) rc = encode_tmap_f32_sw128(&tb_lo, in_lo, (uint64_t)g.total_lines, N, BBOX, BK);
     if (rc != DSBT_OK) return rc;
-    const size_t smem = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
-    rc = ensure_smem((const void*)k_contract_tf32x3, smem);
-    if (rc) return rc;
-    int dev = 0, nsm = 0;
-    DSBT_CUDA_TRY(cudaGetDevice(&dev));
-    DSBT_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int grid = ts.total < nsm ? ts.total : nsm;
     EpiArgs ep{out_mode, out0, out1, phase, p->knl != nullptr};
-    const CUtensorMap& ahi = dir > 0 ? p->tm_T_hi : p->tm_Tt_hi;
-    const CUtensorMap& alo = dir > 0 ? p->tm_T_lo : p->tm_Tt_lo;
-    DSBT_CUDA_TRY(cudaMemsetAsync(sched, 0, sizeof(int), st));
-    ProfScope ps(kKContractTF32, st);
-    k_contract_tf32x3<<<grid, NTHREADS, smem, st>>>(ahi, alo, tb_hi, tb_lo, g, ts, N, dir, ep, p->status,
-                                                    p->spin_limit, sched);
-    DSBT_CUDA_TRY(cudaGetLastError());
-    return DSBT_OK;
+    // Tiles of 128 lines and three stages unless they cut more than a fourth of the
+    // 256-line tiles in two.  A tile's K blocks wait for their loads with two stages:
+    // complex lines of all m at N = 1024, l <= 16 x 2 (136 or 144 tiles, 132 lines at
+    // most) 48.6 us with 256 lines and 42.3 us with 128, N = 4096, l < 32 557 and
+    // 469 us; where tiles fill, the factors are read twice as often: N = 1024, l < 32 x 4
+    // (384 or 640 tiles) 114 and 118 us.  Tiles of 64 lines and four stages are no
+    // faster than 128 even where every group fits them.
+    const auto go = 4 * column_tiles(g, 128) <= 5 * column_tiles(g, BN_MAX) ? launch<128> : launch<BN_MAX>;
+    return go(p, g, dir, tb_hi, tb_lo, ep, sched, st);
 }
 
 }  // namespace dsbt

@@ -1,6 +1,6 @@
 """Interval-scheme contractions (fast_split.cu) take column tiles of 64, 128 or 256
-lines by the largest group, and 64-row or 256-row boxes by a tile's lines; the
-FP16-pair split of caller data (capi.cu) takes 16-byte or 4-byte loads by the
+lines by the groups' sizes, and 64-row or 256-row boxes by a tile's lines; dense
+contractions (gemm_tf32x3.cu) tiles of 128 or 256 lines; the FP16-pair split of caller data (capi.cu) takes 16-byte or 4-byte loads by the
 pointer.  A channel's sums are formed in the same order in each, so its result is
 the same bits."""
 import pytest
@@ -18,8 +18,9 @@ def channels(n, N, dtype):
 @pytest.mark.parametrize("N", [256, 1280, 2048])
 @pytest.mark.parametrize("dtype,sizes", [(torch.float32, (1, 63, 64, 65, 128, 129, 192, 193, 256, 257)),
                                          (torch.complex64, (1, 32, 33, 64, 65, 96, 97, 128, 129))])
-def test_result_independent_of_column_tiles(lib, N, dtype, sizes):
-    plan = lib.Plan(N, 0.1 * N, 3, tf32x3=False, fast_split=True)
+@pytest.mark.parametrize("fast", [True, False])
+def test_result_independent_of_column_tiles(lib, N, dtype, sizes, fast):
+    plan = lib.Plan(N, 0.1 * N, 3, tf32x3=not fast, fast_split=fast)
     x = channels(321, N, dtype)
     b = plan.forward(3, x)
     y = plan.inverse(3, b)
