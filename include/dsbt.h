@@ -76,12 +76,13 @@ extern "C" {
 #define DSBT_PLAN_KCORR 4  /* kinetic phase with the corrected momenta k_nl (Sec. 3,
                               Eq. (kcorr)) instead of k~_n (see dsbt_plan_get_k) */
 #define DSBT_PLAN_FAST64 8 /* with DSBT_PLAN_FP64, N / 64 a power of two: FP64
-                              contractions on planar lines (the kinetic step, the
-                              TDSE) in O(N l log N) work instead of N^2/2: rows of
+                              contractions (grouped calls, the kinetic step, the
+                              TDSE, bound states) in O(N l log N) work instead of N^2/2: rows of
                               T_l are polynomials in m left of the diagonal, applied
                               through a tree of interval moments in orthonormal
                               polynomial bases (stable counterpart of Sec. 2.6).
-                              Extra memory: 8 B x 64 x (l_max+1) x N x log2(N/64)
+                              Extra memory: about
+                              16 B x 64 x (l_max+1) x N x (log2(N/64) + 1)
                               of plan data; FP64 workspaces grow by about
                               8 B x 128 x (N/64) per line. */
 #define DSBT_PLAN_FAST_SPLIT 16 /* any plan grid (N / 128 leaves of 128 rows):

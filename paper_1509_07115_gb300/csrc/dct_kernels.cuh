@@ -32,8 +32,9 @@
 // fixed at compile time (NS = N): every padded shared-memory index is then
 // one base per thread plus constant offsets (all index steps are multiples of
 // 16), which removes most of the integer work of the stages.  The FP32 kernels
-// of the split-FP16 path have one instantiation per plan grid; the FP64 and
-// TF32-split kernels for N = 2048, 4096, 8192 and per Q otherwise.
+// of the split-FP16 path have one instantiation per plan grid; the TF32-split
+// kernels for N = 2048, 4096, 8192 and per Q otherwise; the FP64 kernels per
+// Q > 1 (FP64 on power-of-two grids: dct64.cu).
 #pragma once
 
 #include <math.h>
@@ -345,11 +346,11 @@ template <> __device__ __forceinline__ void st_pair<double2>(double2* p, double2
 // Lines per CTA: as many lines of N/16 threads as fit in 256 threads (one
 // line of up to 512 threads when N/16 > 256), but no more than leave every SM
 // a CTA.  The FP64 transform is bound by the FP64 pipe (1.7 lanes per clock
-// and SM measured: about 48 operations per point, 30 us for a line of 2048
-// points on one SM), so a call of few channels is as slow as its fullest CTA:
-// 64 channels of 2048 points took 67 us with two lines per CTA and 33 us with
-// one, 32 channels of 1024 points 66 us (four per CTA) and 30 us.  Calls with
-// more channels than SMs keep the fuller CTAs.
+// and SM measured: about 48 operations per point), so a call of few channels is
+// as slow as its fullest CTA: with these kernels 64 channels of 2048 points took
+// 67 us with two lines per CTA and 33 us with one (power-of-two grids in FP64 now
+// spread a line over several CTAs, dct64.cu).  Calls with more channels than SMs
+// keep the fuller CTAs.
 inline int lines_per_cta(int N, int nchan) {
     const int most = (N / 16 >= 256) ? 1 : 256 / (N / 16);
     const int even = (nchan + kSMs - 1) / kSMs;
