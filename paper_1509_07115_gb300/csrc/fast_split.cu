@@ -140,7 +140,7 @@ struct FtcSpace {
     int slot_off[MAX_LEVELS + 1];  // first slot of level j
     int npairs;                    // MOMENTS / WEIGHTS tiles of a unit: slot pairs (b = -1: single slot)
     int pair_a[MAX_FSLOTS], pair_b[MAX_FSLOTS];
-    // A unit is one column tile (BN_MAX lines) of one group.  Units are numbered
+    // A unit is one column tile of one group.  Units are numbered
     // group by group (largest l first); unit u's first-kind tiles come before
     // its second-kind tiles, which read what they wrote, and the launch runs
     // block k = [first kind of unit k] [second kind of unit k - lag], so the
@@ -414,8 +414,8 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 }
 
 // The kernel: roles and bounded waits as in gemm_tf32x3.cu; what differs is
-// where each K block comes from, the two kinds of tiles in one launch and the
-// two alternating accumulator buffers.
+// where each K block comes from, the two kinds of tiles in one launch, the two
+// alternating accumulator buffers and the warp that prepares the tiles.
 template <int BN_>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_contract_ftc(const __grid_constant__ CUtensorMap tmA0_hi, const __grid_constant__ CUtensorMap tmA0_lo,
