@@ -269,7 +269,8 @@ int launch64(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const
              cudaStream_t st) {
     using C = Columns<N, CL, EPT>;
     const Kernel64 k = fwd ? (Kernel64)k_dct64_fwd<N, CL, EPT> : (Kernel64)k_dct64_inv<N, CL, EPT>;
-    const size_t smem = 2 * (size_t)C::LEN * sizeof(double2);
+    constexpr size_t smem = 2 * (size_t)C::LEN * sizeof(double2);
+    static_assert(smem <= 227 * 1024, "the two buffers of a CTA's columns");
     if (smem > 48 * 1024)
         if (int rc = ensure_smem((const void*)k, smem)) return rc;
     cudaLaunchConfig_t cfg{};
@@ -288,8 +289,10 @@ int launch64(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const
     return DSBT_OK;
 }
 
-// As many CTAs a line as still have an SM each and 128 threads.  EPT is fixed per
-// grid, so a channel's bits do not depend on how many channels a call has.
+// As many CTAs a line as still have an SM each and 128 threads, and at least as many
+// as hold the line's two buffers: 278 KB at N = 8192, so two there for any number of
+// channels.  EPT is fixed per grid, so a channel's bits do not depend on how many
+// channels a call has.
 template <int N>
 int launch_n(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in, double* out,
              cudaStream_t st) {
@@ -301,7 +304,7 @@ int launch_n(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const
         if (4 * n <= kSMs) return launch64<N, 4, EPT>(fwd, p, g, cplx, in, out, st);
     if constexpr (T >= 256)
         if (2 * n <= kSMs) return launch64<N, 2, EPT>(fwd, p, g, cplx, in, out, st);
-    return launch64<N, 1, EPT>(fwd, p, g, cplx, in, out, st);
+    return launch64<N, N >= 8192 ? 2 : 1, EPT>(fwd, p, g, cplx, in, out, st);
 }
 
 }  // namespace
