@@ -95,7 +95,7 @@ constexpr int AHEAD = 1;
 constexpr int A_BYTES = BM * BK * 2;               // 16 KiB
 constexpr float kFacScale = 16384.f;               // plan factors are stored times 2^14
 constexpr float kFacUnscale = 1.f / 16384.f;
-// Column tile of a launch: 256, 128 or 64 lines (rule in contract_split_fast); the smaller
+// Column tile of a launch: 256, 128 or 64 lines (rule in column_width); the smaller
 // stages buy more of them (192 KB in each case).
 template <int BN_>
 struct TileForm {
@@ -1165,14 +1165,18 @@ void ftc_free(dsbt_plan* p) {
 
 // Augmented lines (an FP16 pair of NAF values per line), then the counter
 // block of a launch: scheduler, abort word and one counter per unit (a unit
-// is a column tile of BN_MAX lines of one group).
+// is a column tile of one group).
 static size_t ftc_aug_bytes(const dsbt_plan* p, size_t lines) {
     return (2 * lines * (size_t)p->ftc->NAF * sizeof(__half) + 255) & ~(size_t)255;
 }
 
+// Unit counters of a call's scratch: as many as tiles of BN_MAX lines can be (a group of
+// n lines has at most n / BN_MAX + 1).  column_width keeps the other widths within it.
+static size_t max_units(size_t lines) { return lines / BN_MAX + kMaxGroups + 1; }
+
 size_t ftc_scratch_bytes(const dsbt_plan* p, size_t lines) {
     if (!p->ftc) return 0;
-    return ftc_aug_bytes(p, lines) + sizeof(int) * (kCtrUnits + lines / BN_MAX + kMaxGroups + 1);
+    return ftc_aug_bytes(p, lines) + sizeof(int) * (kCtrUnits + max_units(lines));
 }
 
 void ftc_set_lag(dsbt_plan* p, int lag) {
@@ -1180,6 +1184,24 @@ void ftc_set_lag(dsbt_plan* p, int lag) {
 }
 
 namespace {
+
+// Column tiles of a launch: 64 lines when every group fits one (a unit a group); 128 unless
+// they are more than 7/5 of the 256-line tiles (three stages instead of two against more
+// reads of the factors; complex lines of all m, 256 -> 128: N = 2048, l <= 33 with 34 -> 36
+// tiles a row 80 -> 69 us, l <= 45 with 46 -> 60 tiles 110 -> 103 us, l <= 40 x 2 with
+// 50 -> 75 tiles 133 us both) or than the scratch has counters, which takes many groups
+// of a little more than 128 lines among small ones.
+int column_width(const GroupTable& g, size_t lines) {
+    int most = 0, t256 = 0, t128 = 0;
+    for (int i = 0; i < g.ngroups; ++i) {
+        const int nl = g.line0[i + 1] - g.line0[i];
+        most = std::max(most, nl);
+        t256 += (nl + 255) / 256;
+        t128 += (nl + 127) / 128;
+    }
+    if (most <= 64) return 64;
+    return 5 * t128 <= 7 * t256 && (size_t)t128 <= max_units(lines) ? 128 : BN_MAX;
+}
 
 // One launch over the groups (largest l first): the first kind (MOMENTS or
 // WEIGHTS) and the second (EVAL or LEAFOUT) of every unit, interleaved.
@@ -1218,7 +1240,7 @@ int launch_fused(const dsbt_plan* p, const GroupTable& g, int dir, const CUtenso
     }
     fs.units = fs.u0[g.ngroups];
     if (fs.units == 0) return DSBT_OK;
-    if ((size_t)fs.units > lines / BN_MAX + kMaxGroups + 1) {
+    if ((size_t)fs.units > max_units(lines)) {
         set_error("interval-scheme contraction: unit counters exceed the scratch");
         return DSBT_ERR_INVALID;
     }
@@ -1271,19 +1293,8 @@ int contract_split_fast(const dsbt_plan* p, const GroupTable& g, int dir, const 
     if (rc == DSBT_OK) rc = encode_tmap_f16_sw128(&augs_l, aug_lo, R, NA, BBOX_S, BK);
     if (rc != DSBT_OK) return rc;
     const EpiArgs ep{out_mode, out0, out1, phase, p->knl != nullptr, scale, aug_hi, aug_lo, NA};
-    // Column tiles: 64 lines when every group fits one; 128 unless they are more than
-    // 7/5 of the 256-line tiles (three stages instead of two against more reads of the
-    // factors; complex lines of all m, 256 -> 128: N = 2048, l <= 33 with 34 -> 36 tiles
-    // a row 80 -> 69 us, l <= 45 with 46 -> 60 tiles 110 -> 103 us, l <= 40 x 2 with
-    // 50 -> 75 tiles 133 us both).
-    int most = 0, t256 = 0, t128 = 0;
-    for (int i = 0; i < g.ngroups; ++i) {
-        const int nl = g.line0[i + 1] - g.line0[i];
-        most = std::max(most, nl);
-        t256 += (nl + 255) / 256;
-        t128 += (nl + 127) / 128;
-    }
-    const auto launch = most <= 64 ? launch_fused<64> : (5 * t128 <= 7 * t256 ? launch_fused<128> : launch_fused<BN_MAX>);
+    const int bn = column_width(g, R);
+    const auto launch = bn == 64 ? launch_fused<64> : (bn == 128 ? launch_fused<128> : launch_fused<BN_MAX>);
     if (dir > 0)
         return launch(p, g, dir, f->tm_qT_hi, f->tm_qT_lo, f->tm_D_hi, f->tm_D_lo, in_h, in_l, f->tm_bA_hi, f->tm_bA_lo,
                       aug_h, aug_l, f->tm_D_hi, f->tm_D_lo, ins_h, ins_l, augs_h, augs_l, ep, ctr, R, st);
