@@ -70,12 +70,17 @@ __device__ __forceinline__ void fixed_b(double v, int ef, uint32_t& lo, uint32_t
     fixed_point(vl, mh, 1 + ef - (int)((vh >> 20) & 0x7ffu), (int)vh >> 31, lo, hi);
 }
 
+// The smallest scale taken: the unit of to_double is then the smallest number 2^-1074,
+// and every such number a multiple of 2^(E - 62).  (With the scale of 2^-1020 and below
+// that unit underflowed, and the line's results were zeros.)
+constexpr int kMinScale = 3;
+
 // The same for any scale: a line whose largest magnitude is below 2^-958.
 static __device__ __noinline__ void fixed_b_tiny(double v, int ef, uint32_t& lo, uint32_t& hi) {
     const uint32_t vl = (uint32_t)__double2loint(v), vh = (uint32_t)__double2hiint(v);
     const int e = (int)((vh >> 20) & 0x7ffu);
     const uint32_t mh = (__funnelshift_l(vl, vh, 10) & 0x3fffffffu) | (e ? 0x40000000u : 0u);
-    fixed_point(vl, mh, 1 + max(ef, 1) - max(e, 1), (int)vh >> 31, lo, hi);
+    fixed_point(vl, mh, 1 + max(ef, kMinScale) - max(e, 1), (int)vh >> 31, lo, hi);
 }
 
 // Digit d of two fixed-point words as a pair of FP16 integers: byte b becomes
@@ -200,7 +205,7 @@ __device__ __forceinline__ int exponent4(const double* v) {
 __device__ __forceinline__ double to_double(long long hi, long long lo, int ef) {
     if (ef == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);   // a line with an infinity or NaN
     const long long v = hi * (1ll << 20) + ((lo + 2048) >> 12);
-    const int e = max(ef, 1) - 1022 - 55;
+    const int e = max(ef, kMinScale) - 1022 - 55;
     const double s = e > -1022 ? __hiloint2double((e + 1023) << 20, 0) : ldexp(1.0, e);
     return (double)v * s;
 }
