@@ -1129,7 +1129,7 @@ extern "C" int dsbt_batch_create_ex(int ntrans, const int* N, const int* l_max, 
         if (!rc) rc = encode_tmap_f32_sw128(&cm[d].m[2], ih, (uint64_t)b->L * Nd, CROWS, BM, 32);
         if (!rc) rc = encode_tmap_f32_sw128(&cm[d].m[3], il, (uint64_t)b->L * Nd, CROWS, BM, 32);
         if (rc) { batch_free(b); return rc; }
-        if (cudaStreamSynchronize(st) != cudaSuccess) { batch_free(b); set_error("per-N table build failed"); return DSBT_ERR_CUDA; }
+        if (cudaStreamSynchronize(st) != cudaSuccess) { batch_free(b); cudaGetLastError(); set_error("per-N table build failed"); return DSBT_ERR_CUDA; }
     }
     cudaFree(b->comp64);
     b->comp64 = nullptr;
@@ -1297,7 +1297,10 @@ extern "C" int dsbt_batch_capture_kinetic(const dsbt_batch* b, double tau, const
     }
     if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
-    if (rc) return rc;
+    if (rc) {
+        cudaGetLastError();
+        return rc;
+    }
     *graph_exec = (void*)ge;
     return DSBT_OK;
 }

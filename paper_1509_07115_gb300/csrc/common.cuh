@@ -14,10 +14,13 @@ namespace dsbt {
 
 void set_error(const char* fmt, ...);
 
+// A failed call also leaves its code as the thread's last error, which the check after
+// the next launch would report as that launch's: it is taken back here.
 #define DSBT_CUDA_TRY(expr)                                                            \
     do {                                                                               \
         cudaError_t e__ = (expr);                                                      \
         if (e__ != cudaSuccess) {                                                      \
+            (void)cudaGetLastError();                                                  \
             ::dsbt::set_error("%s:%d: %s: %s", __FILE__, __LINE__, #expr,              \
                               cudaGetErrorString(e__));                                \
             return DSBT_ERR_CUDA;                                                      \

@@ -395,6 +395,7 @@ extern "C" int dsbt_plan_create(int N, double r_max, int l_max, int flags, void*
     }
     if (cudaMemsetAsync(p->status, 0, sizeof(unsigned), st) != cudaSuccess) {
         plan_free(p);
+        cudaGetLastError();
         set_error("dsbt_plan_create: memset failed");
         return DSBT_ERR_CUDA;
     }
@@ -403,6 +404,7 @@ extern "C" int dsbt_plan_create(int N, double r_max, int l_max, int flags, void*
         kcorr_table(N, r_max, l_max, k);
         if (cudaMemcpy(p->knl, k.data(), k.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
             plan_free(p);
+            cudaGetLastError();
             set_error("dsbt_plan_create: momentum table upload failed");
             return DSBT_ERR_CUDA;
         }

@@ -102,6 +102,7 @@ int run_streamed(int which, const dsbt_plan* p, const int* counts, int dtype, do
     if (cudaStreamCreateWithFlags(&s_in, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&s_out, cudaStreamNonBlocking) != cudaSuccess) {
         cleanup();
+        cudaGetLastError();
         set_error("stream creation failed");
         return DSBT_ERR_CUDA;
     }
@@ -110,6 +111,7 @@ int run_streamed(int which, const dsbt_plan* p, const int* counts, int dtype, do
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
             e = nullptr;
             cleanup();
+            cudaGetLastError();
             set_error("event creation failed");
             return DSBT_ERR_CUDA;
         }
@@ -154,6 +156,7 @@ int run_streamed(int which, const dsbt_plan* p, const int* counts, int dtype, do
     }
     cleanup();
     if (ce != cudaSuccess) {
+        cudaGetLastError();
         set_error("streamed transform: %s", cudaGetErrorString(ce));
         return DSBT_ERR_CUDA;
     }
