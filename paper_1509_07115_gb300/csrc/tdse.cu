@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(128) k_tdse_potential(const double2* x, double
     if (tid < 4 * TI) sh.ef[tid / (2 * TI)][tid % (2 * TI)] = 0;
     if (tid < TI) {
         double sn, cs;
-        sincos(-(e2 >= 0 ? 2.0 : 1.0) * V[i] * ht, &sn, &cs);
+        sincos(-V[i] * (e2 >= 0 ? 2.0 * ht : ht), &sn, &cs);   // 2 V may pass the largest number
         sh.vph[t] = make_double2(cs, sn);
     }
     for (int k = tid; k < (L16 - L) * TI; k += blockDim.x) sh.grid[L + k / TI][k % TI] = make_double2(0.0, 0.0);

@@ -257,7 +257,8 @@ __global__ void __launch_bounds__(128) k_tdse3d_potential(const double2* x, doub
     for (int k = tid; k < L * TI3; k += blockDim.x) {
         const int j = k / TI3, i = i0 + k % TI3;
         double sn, c;
-        sincos(-((f2 >= 0 ? 2.0 : 1.0) * V[i] + rr[i] * f[2] * a.eta[j]) * ht, &sn, &c);
+        // (w V + r F_z eta) ht with the w at ht: 2 V may pass the largest number
+        sincos(-(V[i] + (f2 >= 0 ? 0.5 : 1.0) * rr[i] * f[2] * a.eta[j]) * (f2 >= 0 ? 2.0 * ht : ht), &sn, &c);
         zph[k] = make_double2(c / NM, sn / NM);
     }
     if (tid < TI3) rad[tid] = rr[i0 + tid];
