@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
     };
     if (NARROW) {
         const int j = tq & 1, r = m * 16 + gr + 4 * (tq & 2);
-        double v = to_double(shi[0], slo[0], ef[j]);
+        double v = to_double_once(shi[0], slo[0], ef[j]);
         if (ph) {   // the lane's neighbour holds the channel's other part
             const double o = __shfl_xor_sync(0xffffffffu, v, 1);
             const double2 w = phase_of(r);
@@ -607,9 +607,9 @@ __global__ void __launch_bounds__(THREADS, NL_ == 2 ? 4 : 3) k_mm64(const __grid
             const int j = n * 8 + 2 * tq;
             if (j >= nline) continue;
             const int e0 = ef[j], e1 = ef[j + 1];
-            put(j, m * 16 + gr, to_double(shi[n * 4], slo[n * 4], e0), to_double(shi[n * 4 + 1], slo[n * 4 + 1], e1));
-            put(j, m * 16 + gr + 8, to_double(shi[n * 4 + 2], slo[n * 4 + 2], e0),
-                to_double(shi[n * 4 + 3], slo[n * 4 + 3], e1));
+            put(j, m * 16 + gr, to_double_once(shi[n * 4], slo[n * 4], e0), to_double_once(shi[n * 4 + 1], slo[n * 4 + 1], e1));
+            put(j, m * 16 + gr + 8, to_double_once(shi[n * 4 + 2], slo[n * 4 + 2], e0),
+                to_double_once(shi[n * 4 + 3], slo[n * 4 + 3], e1));
         }
     }
 }

@@ -201,13 +201,34 @@ __device__ __forceinline__ int exponent4(const double* v) {
 
 // A result: sum = 2^(E - 67) (hi 2^32 + lo).  |sum| <= ||a|| ||x|| < 2^(E + 6.5)
 // for K <= 8192, so hi 2^20 stays below 2^62 and one 64-bit integer with the
-// unit 2^(E - 55) holds it.
+// unit 2^(E - 55) holds it: an error of 2^-56 of the line's scale in every result.
 __device__ __forceinline__ double to_double(long long hi, long long lo, int ef) {
     if (ef == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);   // a line with an infinity or NaN
     const long long v = hi * (1ll << 20) + ((lo + 2048) >> 12);
     const int e = max(ef, kMinScale) - 1022 - 55;
     const double s = e > -1022 ? __hiloint2double((e + 1023) << 20, 0) : ldexp(1.0, e);
     return (double)v * s;
+}
+
+// v 2^e for e <= -1022, where 2^e may be no FP64 number (a line whose largest magnitude is
+// below 2^-955): in two steps, of which only the second rounds.
+static __device__ __noinline__ double times_small_power(double v, int e) {
+    return v * __hiloint2double((e + 1223) << 20, 0) * 0x1p-200;
+}
+
+// The same rounded to FP64 once, for long lines: with lo's carry in it hi has at most 42
+// bits, and the whole, shifted down by the s of them above 31 that it has, fills a 64-bit
+// integer.  (The unit above, in the N results of a line with one large entry, is
+// sqrt(N / 3) 2^-56 of it: 1.5e-15 at N = 8192, three times the sine transform's error.
+// The columns of the angular products have 64 entries, 6e-17, and keep it.)
+__device__ __forceinline__ double to_double_once(long long hi, long long lo, int ef) {
+    if (ef == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
+    hi += lo >> 32;
+    const int top = (int)(hi >> 31), s = 32 - __clz(top ^ (top >> 31));
+    const long long v = (long long)((unsigned long long)hi << (32 - s)) + (long long)((uint32_t)lo >> s);
+    const int e = max(ef, kMinScale) - 1022 - 67 + s;
+    if (e <= -1022) return times_small_power((double)v, e);
+    return (double)v * __hiloint2double((e + 1023) << 20, 0);
 }
 
 }  // namespace mm64
