@@ -56,7 +56,7 @@ int dct_forward_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const do
     int rc = launch_cfg(k, p->N, nchannels(g), sizeof(double2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctFwd, st);
-    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, nullptr, nullptr, p->tw64, p->post64, fwd_scale<double>(p->N));
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, nullptr, nullptr, p->tw64, p->post64, fwd_scale(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -70,7 +70,7 @@ int dct_forward_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
     int rc = launch_cfg(k, p->N, nchannels(g), sizeof(float2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctFwd, st);
-    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, nullptr, p->tw32, p->post32, fwd_scale<float>(p->N));
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, nullptr, p->tw32, p->post32, {});
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -88,7 +88,7 @@ int dct_inverse_f64(const dsbt_plan* p, const GroupTable& g, bool cplx, const do
     int rc = launch_cfg(k, p->N, nchannels(g), sizeof(double2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctInv, st);
-    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw64, p->post64, inv_scale<double>(p->N));
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw64, p->post64, inv_scale(p->N));
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }

@@ -285,7 +285,7 @@ int launch64(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const
     cfg.attrs = at;
     cfg.numAttrs = CL > 1 ? 1 : 0;
     DSBT_CUDA_TRY(cudaLaunchKernelEx(&cfg, k, g, cplx ? 1 : 0, in, out, (const double2*)p->tw64,
-                                     (const double2*)p->post64, fwd ? fwd_scale<double>(N) : inv_scale<double>(N)));
+                                     (const double2*)p->post64, fwd ? fwd_scale(N) : inv_scale(N)));
     return DSBT_OK;
 }
 

@@ -48,7 +48,7 @@ int dct_forward_f16(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
     int rc = launch_cfg(k, p->N, nchannels(g), sizeof(float2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctFwd, st);
-    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, scale, p->tw32, p->post32, fwd_scale<float>(p->N));
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out_hi, out_lo, scale, p->tw32, p->post32, {});
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }
@@ -62,7 +62,7 @@ int dct_inverse_f32(const dsbt_plan* p, const GroupTable& g, bool cplx, const fl
     int rc = launch_cfg(k, p->N, nchannels(g), sizeof(float2), nb, th, sm);
     if (rc) return rc;
     ProfScope ps(kKDctInv, st);
-    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw32, p->post32, inv_scale<float>(p->N));
+    k<<<nb, th, sm, st>>>(g, p->N, cplx ? 1 : 0, in, out, p->tw32, p->post32 + p->N, {});
     DSBT_CUDA_TRY(cudaGetLastError());
     return DSBT_OK;
 }

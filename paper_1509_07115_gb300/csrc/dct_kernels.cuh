@@ -367,12 +367,17 @@ inline int lines_per_cta(int N, int nchan) {
 // subnormal step (2^-24) 2^-36 below the channel norm.
 enum : int { kPlain = 0, kSplitTF32 = 1, kSplitF16 = 2 };
 
-// Scale factors of a transform, computed on the host: as per-thread square
-// roots and divisions in FP64 they cost as much as a radix-4 stage.
+// Scale factors of an FP64 transform, computed on the host: as per-thread square
+// roots and divisions in FP64 they cost as much as a radix-4 stage.  FP32 transforms
+// have them in their post-twiddle tables (k_twiddles, plan.cu), formed in FP64: a factor
+// rounded to FP32 is up to 6e-8 off, alike for every output, where the entries of a
+// table round each for itself (inverse at N = 6400: error 6.0e-7 -> 5.5e-7).
 template <typename R>
 struct DctScale {
     R c0, c1;   // forward: sqrt(1/N), sqrt(2/N); inverse: 1/sqrt(N), 1/sqrt(2N), the unscaled FFT's 1/N in them
 };
+template <>
+struct DctScale<float> {};
 
 // Power-of-two exponent e with x 2^e in [2^12, 2^13) (0 for 0, inf, nan).
 __device__ __forceinline__ int scale_exp(float nrm) {
@@ -461,7 +466,6 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
     __shared__ C sroot[32];
     fft_stages<Q, NS>(s, tw, sroot, N, lt, T, 1, N);
     if (!live) return;
-    const R sc1 = dsc.c1, sc0 = dsc.c0;
     const int line = g.line0[gi] + (cplx ? 2 * local : local);
     float fs = 1.f;
     if (MODE == kSplitF16) {
@@ -474,7 +478,8 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
             if (cplx) scale[line + 1] = ldexpf(1.f, -e);
         }
     }
-    if (MODE == kPlain) {
+    if constexpr (MODE == kPlain) {   // FP64
+        const R sc1 = dsc.c1, sc0 = dsc.c0;
         // k and N - k together: with A = w V_k and B = conj(w) V_{N-k} (w_{N-k} =
         // -i conj(w)), X_k = (A + B) / 2 and X_{N-k} = i (A - B) / 2: two
         // products for two outputs, and half the shared-memory reads.
@@ -523,13 +528,10 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_fwd(GroupTa
             // V_k and V_{N-k} (V_0 for k = 0)
             const C a = NS > 0 ? s[padi(2 * lt + e) + i * st2] : s[padi(k)];
             const C b = (k == 0) ? a : (NS > 0 ? s[padi(N - 2 * lt - e) - i * st2] : s[padi(N - k)]);
-            const C w = post[k];
-            C v;   // 1/2 (w a + conj(w) b)
-            v.x = (R)0.5 * ((w.x * a.x - w.y * a.y) + (w.x * b.x + w.y * b.y));
-            v.y = (R)0.5 * ((w.x * a.y + w.y * a.x) + (w.x * b.y - w.y * b.x));
-            const R sc = (k == 0) ? sc0 : sc1;
-            v.x *= sc;
-            v.y *= sc;
+            const C w = post[k];   // FP32: the 1/2 and the scale are in the table
+            C v;   // w a + conj(w) b
+            v.x = (w.x * a.x - w.y * a.y) + (w.x * b.x + w.y * b.y);
+            v.y = (w.x * a.y + w.y * a.x) + (w.x * b.y - w.y * b.x);
             X[e] = v;
         }
         // storage index of k: odd l -> k; even l -> N-1-k (pairs stay adjacent, order flips)
@@ -639,8 +641,10 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_dct_inv(GroupTa
         t.x = a.x + b.y;
         t.y = a.y - b.x;
         C w = post[k];
-        const R sc = (k == 0) ? dsc.c0 : dsc.c1;
-        w.x *= sc; w.y *= sc;
+        if constexpr (sizeof(R) == 8) {
+            const R sc = (k == 0) ? dsc.c0 : dsc.c1;
+            w.x *= sc; w.y *= sc;
+        }
         const C v = cmulc(t, w);
         vk[u].x = v.x;
         vk[u].y = -v.y;
@@ -682,16 +686,12 @@ inline int launch_cfg(K kernel, int N, int nchan, size_t elem, unsigned& blocks,
     return DSBT_OK;
 }
 
-template <typename R>
-inline DctScale<R> fwd_scale(int N) {
-    return {(R)sqrt(1.0 / (double)N), (R)sqrt(2.0 / (double)N)};
-}
+inline DctScale<double> fwd_scale(int N) { return {sqrt(1.0 / (double)N), sqrt(2.0 / (double)N)}; }
 // 1/sqrt(N), 1/sqrt(2N) as the reciprocals of the rounded forward factors times
 // N, so that a forward and an inverse transform scale by one as nearly as can be.
-template <typename R>
-inline DctScale<R> inv_scale(int N) {
-    const DctScale<R> f = fwd_scale<R>(N);
-    return {(R)(1.0 / ((double)f.c0 * N)), (R)(1.0 / ((double)f.c1 * N))};
+inline DctScale<double> inv_scale(int N) {
+    const DctScale<double> f = fwd_scale(N);
+    return {1.0 / (f.c0 * N), 1.0 / (f.c1 * N)};
 }
 
 // Odd part Q of q = N / 256; every N = 256 q with q <= 32 has Q in 1..31.

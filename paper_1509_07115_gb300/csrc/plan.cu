@@ -197,7 +197,9 @@ __global__ void k_twiddles(double2* tw64, double2* post64, float2* tw32, float2*
     tw32[t] = make_float2((float)c, (float)s);
     sincospi(-(double)t / (2.0 * (double)N), &s, &c);
     post64[t] = make_double2(c, s);
-    post32[t] = make_float2((float)c, (float)s);
+    const double f = sqrt((t == 0 ? 1.0 : 2.0) / (double)N), i = 1.0 / (f * (double)N);
+    post32[t] = make_float2((float)(0.5 * f * c), (float)(0.5 * f * s));
+    post32[N + t] = make_float2((float)(i * c), (float)(i * s));
 }
 
 // ------------------------------------------------------------------ host side
@@ -296,7 +298,7 @@ int plan_twiddles_only(int N, double r_max, cudaStream_t st, dsbt_plan** out) {
     bool ok = cudaMalloc((void**)&p->tw64, N * sizeof(double2)) == cudaSuccess &&
               cudaMalloc((void**)&p->post64, N * sizeof(double2)) == cudaSuccess &&
               cudaMalloc((void**)&p->tw32, N * sizeof(float2)) == cudaSuccess &&
-              cudaMalloc((void**)&p->post32, N * sizeof(float2)) == cudaSuccess;
+              cudaMalloc((void**)&p->post32, 2 * N * sizeof(float2)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         cudaFree(p->tw64); cudaFree(p->post64); cudaFree(p->tw32); cudaFree(p->post32);
@@ -384,7 +386,7 @@ extern "C" int dsbt_plan_create(int N, double r_max, int l_max, int flags, void*
     ok = ok && alloc((void**)&p->tw64, N * sizeof(double2)) &&
          alloc((void**)&p->post64, N * sizeof(double2)) &&
          alloc((void**)&p->tw32, N * sizeof(float2)) &&
-         alloc((void**)&p->post32, N * sizeof(float2)) &&
+         alloc((void**)&p->post32, 2 * N * sizeof(float2)) &&
          alloc((void**)&p->status, sizeof(unsigned));
     if (ok && (flags & DSBT_PLAN_KCORR)) ok = alloc((void**)&p->knl, L * N * sizeof(double));
     if (!ok) {

@@ -31,7 +31,8 @@ struct dsbt_plan {
     float* Tthi;
     float* Ttlo;
     // FFT twiddles w^t = exp(-2 pi i t / N), t < N, and the cosine-transform
-    // post-twiddles exp(-i pi k / (2N)), k < N.
+    // post-twiddles exp(-i pi k / (2N)), k < N.  post32: [0, N) times half the forward
+    // transform's scale, [N, 2N) times the inverse's.
     double2* tw64;
     double2* post64;
     float2* tw32;
