@@ -291,7 +291,7 @@ int launch64(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const
 
 // As many CTAs a line as still have an SM each and 128 threads, and at least as many
 // as hold the line's two buffers: 278 KB at N = 8192, so two there for any number of
-// channels.  EPT is fixed per grid, so a channel's bits do not depend on how many
+// channels (100: 134 / 142 us, 1000: 899 / 957 us).  EPT is fixed per grid, so a channel's bits do not depend on how many
 // channels a call has.
 template <int N>
 int launch_n(bool fwd, const dsbt_plan* p, const GroupTable& g, bool cplx, const double* in, double* out,

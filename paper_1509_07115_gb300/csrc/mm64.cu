@@ -21,7 +21,7 @@
 // forms their digits there (each A entry is used by one warp): from doubles, or
 // for the interval scheme's operands from fixed-point words made at plan
 // creation.  The lines are copied to shared memory and turned into digits there,
-// once per CTA, 64 columns at a time.
+// once per CTA, 128 (wide) or 512 (narrow) columns at a time.
 // Each line's scale is its largest exponent over the K range of the tile, found
 // in a first pass over the (cached) lines, so no scale travels between kernels.
 // The range depends on the row's block of 64 only and the sums are exact, so a
@@ -30,7 +30,8 @@
 //
 // Two forms by the number of real lines of a group:
 //   wide    16 lines a tile, one matrix instruction of 8 lines per digit pair:
-//           bound by the tensor pipe, 72 clocks per 16 x 16 x 8 lines
+//           held by the matrix instructions (72 clocks per 16 x 16 x 8 lines, 28 to
+//           39 % of the tensor pipe's cycles) and the conversions beside them
 //   narrow  2 lines a tile, the 8 digits of both lines as 16 columns, so one
 //           digit of A meets all digits of the lines in two instructions (12
 //           instead of 36): bound by turning A into digits and by reading it
@@ -41,7 +42,7 @@
 //
 // Measured on a GB300, forward + inverse contraction of one call (before: FP64
 // multiply-adds on the same schemes):
-//   interval scheme, N = 2048, l < 32 all m (2048 lines)   4.66 -> 0.69 ms
+//   interval scheme, N = 2048, l < 32 all m (2048 lines)   4.66 -> 0.71 ms
 //   interval scheme, N = 2048, l < 40, 34 lines each       1.88 -> 0.55 ms
 //   interval scheme, N = 2048, l < 64, 2 lines each        374 -> 233 us
 //   dense, N = 1280, l <= 20 all m (882 lines)             7.25 -> 0.61 ms
@@ -665,8 +666,8 @@ int launch_both(MmArgs a, const GroupTable& g, cudaStream_t st) {
 }  // namespace
 
 // The digits replace FP64 multiply-adds in every call: measured faster from one
-// line of 256 points (N = 256, l <= 9) to 2048 lines of 2048, at errors against
-// 64-bit references that are equal or smaller.
+// line of 256 points (N = 256, l <= 9) to 2048 lines of 2048; for the errors of both see
+// mm64.cuh.
 int contract_f64(const dsbt_plan* p, const GroupTable& g, int dir, const double* in, int in_cplx, double* out,
                  int out_cplx, const double2* phase, cudaStream_t st, double* fast_scratch, const double* row_scale) {
     if (!p->T64) {

@@ -9,12 +9,21 @@
 // most 2^14, so a sum of 2^10 of them is an integer of at most 2^24 and exact
 // in the FP32 accumulator (checked on the hardware for random and extreme
 // digits).  The 36 digit products D_i D_j with i + j <= 7 give
-//     sum_k a_k x_k = sum_s 2^(-8 s) sum_{i + j = s} sum_k D_i(a_k) D_j(x_k)
-// up to terms below 2^-64 of the operands' scales; the sums of each s are added
-// up as 64-bit integers and rounded to FP64 once.  FP64 arithmetic rounds every
-// multiply-add at 2^-53 of the partial sum instead; against 64-bit references
-// the results here are as close or closer (tests/test_mm64.py).  36 matrix
-// instructions of two clocks replace 2048 multiply-adds: 28 per clock and SM.
+//     sum_k a_k x_k = sum_s 2^(-8 s) sum_{i + j = s} sum_k D_i(a_k) D_j(x_k),
+// the sums of each s added up as integers (the results' rounding: to_double,
+// to_double_once).  36 matrix instructions of two clocks replace 2048
+// multiply-adds: 28 per clock and SM.
+//
+// What is left out, with 2 the scale of A and 2^E that of a line x: the bits of an
+// operand below 2^-62 of its scale, and the products with i + j >= 8, which for
+// each k are seven terms of up to 2^-62 of the scales' product (i + j = 8; the next
+// ones 2^-8 of that).  At random digits that is sqrt(K) 2^-61 of 2^E in a sum over K
+// columns.  FP64 multiply-adds round at 2^-53 of each product and partial sum instead: more
+// where a line's entries are alike in size, less where dense factors meet a line with
+// one large entry among small ones (error of the inverse over the norm, a unit entry among
+// entries of 1e-5, here and with multiply-adds: dense N = 1024 5e-16 and 4e-16,
+// N = 2048 8e-16 and 5e-16, N = 4096 1.6e-15 and 6e-16; through the interval scheme, whose
+// sums are short, no difference).
 //
 // K runs in blocks of 16.  Lane (g = lane / 4, t = lane % 4) of a warp holds
 // columns 4t .. 4t+3 of rows g and g + 8 of the A operand (one 32-byte piece of
